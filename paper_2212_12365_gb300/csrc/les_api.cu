@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "les_internal.cuh"
+#include "les_sums.cuh"
 
 using namespace les;
 
@@ -41,7 +42,7 @@ struct JetHost {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-constexpr int DIAG_BLOCKS = 608; // blocks of the diagnostics reduction (fixed order)
+constexpr int DIAG_BLOCKS = SUM_MAX_BLOCKS; // blocks of the diagnostics reduction (scratch size)
 
 } // namespace
 
@@ -285,7 +286,7 @@ static GlobalPlan plan_global(int njets, size_t jetdev_bytes, int nblk_diag, lon
     P.o_dt = take(sizeof(double) * njets);
     P.o_level = take(sizeof(long long));
     P.o_bits = take(sizeof(unsigned long long) * njets);
-    P.o_part = take(sizeof(double) * 17 * nblk_diag);
+    P.o_part = take(sizeof(double) * SUM_PART * nblk_diag);
     P.o_diag = take(sizeof(double) * 16);
     P.o_pbase = take(sizeof(long long));
     P.o_stage = take(sizeof(double) * 5 * (size_t)maxN);
@@ -1171,8 +1172,9 @@ template <typename real> static int diag_impl(les_handle *h, int jet, les_diag *
     int rc = residual_of_jet<real>(h, jet);
     if (rc) return rc;
     const JetDev<real> *jets = (const JetDev<real> *)h->d_jets;
-    Launch<real>::diag_partials(jets, jet, h->d_partials, h->nblk_diag, h->st);
-    launch_diag_final(h->d_partials, h->nblk_diag, h->d_diag, h->st);
+    const int nb = std::min(h->nblk_diag, sum_blocks(h->J[jet].npad));
+    Launch<real>::diag_partials(jets, jet, h->d_partials, nb, h->st);
+    launch_diag_final(h->d_partials, nb, h->d_diag, h->st);
     CK(cudaGetLastError());
     double out[12];
     CK(cudaMemcpyAsync(out, h->d_diag, sizeof(out), cudaMemcpyDeviceToHost, h->st));

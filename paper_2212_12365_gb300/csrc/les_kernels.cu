@@ -13,6 +13,7 @@
 #include <cstdint>
 
 #include "les_internal.cuh"
+#include "les_sums.cuh"
 
 namespace les {
 
@@ -744,93 +745,45 @@ __global__ void __launch_bounds__(BLOCK) k_dt_max(const JetDev<real> *__restrict
 }
 
 // ---------------------------------------------------------------------------
-// Diagnostics: per-block partials in a fixed order, then one block combines.
-// partial layout (NPART = 17 doubles): [0] max|RHS_rho|, [1..5] sum RHS^2,
-// [6..10] Neumaier sums of Qhat, [11..15] their compensations, [16] the
-// count of non-finite state or residual values (reported as out[11]).
+// Diagnostics: per-block partials in a fixed order, then one block combines
+// (les_sums.cuh)
 // ---------------------------------------------------------------------------
 
-constexpr int NPART = 17;
-
-__device__ __forceinline__ void neumaier_add(double &s, double &c, double v)
-{
-    double t = s + v;
-    if (fabs(s) >= fabs(v)) c += (s - t) + v;
-    else c += (v - t) + s;
-    s = t;
-}
-
 template <typename real>
-__global__ void __launch_bounds__(BLOCK) k_diag_partials(const JetDev<real> *__restrict__ jets,
-                                                         int jet, double *partials)
+__global__ void __launch_bounds__(SUM_BLOCK, 4) k_diag_partials(const JetDev<real> *__restrict__ jets,
+                                                                int jet, double *part)
 {
     const JetDev<real> &J = jets[jet];
-    __shared__ double sh[NPART][BLOCK];
-    double mx = 0.0, l2[5] = {0, 0, 0, 0, 0}, s[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0};
-    double bad = 0.0;
-    const long long fs = J.fs;
-    for (long long lp = blockIdx.x * (long long)blockDim.x + threadIdx.x; lp < J.npts_pad;
-         lp += (long long)gridDim.x * blockDim.x) {
-        int q[3];
-        if (!point_of(J, lp, q)) continue;
-        // the Qhat the FP64 store holds (unscaled on a polar axis) from an
-        // unscaled FP32 store
-        const double qs = sizeof(real) == sizeof(float) ? state_scale(J.jinv64[lp]) : 1.0;
-        for (int f = 0; f < 5; ++f) {
-            double r = (double)J.rhs[f * fs + lp];
-            double v = (double)J.q[0][f * fs + lp] * qs;
-            if (!isfinite(r) || !isfinite(v)) bad += 1.0;
-            l2[f] += r * r;
-            neumaier_add(s[f], c[f], v);
-        }
-        mx = fmax(mx, fabs((double)J.rhs[lp]));
-    }
-    sh[0][threadIdx.x] = mx;
-    for (int f = 0; f < 5; ++f) {
-        sh[1 + f][threadIdx.x] = l2[f];
-        sh[6 + f][threadIdx.x] = s[f];
-        sh[11 + f][threadIdx.x] = c[f];
-    }
-    sh[16][threadIdx.x] = bad;
-    __syncthreads();
-    for (int st = BLOCK / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            int o = threadIdx.x + st;
-            sh[0][threadIdx.x] = fmax(sh[0][threadIdx.x], sh[0][o]);
-            for (int f = 0; f < 5; ++f) {
-                sh[1 + f][threadIdx.x] += sh[1 + f][o];
-                double a = sh[6 + f][threadIdx.x], ca = sh[11 + f][threadIdx.x];
-                neumaier_add(a, ca, sh[6 + f][o]);
-                sh[6 + f][threadIdx.x] = a;
-                sh[11 + f][threadIdx.x] = ca + sh[11 + f][o];
-            }
-            sh[16][threadIdx.x] += sh[16][o];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < NPART) partials[blockIdx.x * NPART + threadIdx.x] = sh[threadIdx.x][0];
+    const long long n = J.npts_pad, fs = J.fs;
+    const long long stride = (long long)gridDim.x * SUM_BLOCK;
+    const long long p0 = blockIdx.x * (long long)SUM_BLOCK + threadIdx.x;
+    const int pitch = J.pitch, ni = J.n[0];
+    const real *Q = J.q[0], *R = J.rhs;
+    const double *jinv = J.jinv64;
+    // column of the thread's point, carried from point to point
+    int i = (int)(p0 % pitch);
+    const int di = (int)(stride % pitch);
+    sum_block((n + stride - 1) / stride,
+              [&](long long t, double q[5], double r[5]) {
+                  const long long p = p0 + t * stride;
+                  const bool in = p < n && i < ni; // padding columns hold nothing
+                  i += di;
+                  if (i >= pitch) i -= pitch;
+                  // the Qhat the FP64 store holds (unscaled on a polar axis) from an
+                  // unscaled FP32 store
+                  const double qs = sizeof(real) == sizeof(float) && in ? state_scale(jinv[p]) : 1.0;
+#pragma unroll
+                  for (int f = 0; f < 5; ++f) {
+                      q[f] = in ? (double)Q[f * fs + p] * qs : 0.0;
+                      r[f] = in ? (double)R[f * fs + p] : 0.0;
+                  }
+              },
+              part);
 }
 
-__global__ void k_diag_final(const double *partials, int nblocks, double *out)
+__global__ void __launch_bounds__(SUM_FINAL_THREADS) k_diag_final(const double *part, int nblocks, double *out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double mx = 0.0, l2[5] = {0, 0, 0, 0, 0}, s[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0}, bad = 0;
-    for (int b = 0; b < nblocks; ++b) {
-        const double *P = partials + b * NPART;
-        mx = fmax(mx, P[0]);
-        for (int f = 0; f < 5; ++f) {
-            l2[f] += P[1 + f];
-            neumaier_add(s[f], c[f], P[6 + f]);
-            c[f] += P[11 + f];
-        }
-        bad += P[16];
-    }
-    out[0] = mx;
-    for (int f = 0; f < 5; ++f) {
-        out[1 + f] = sqrt(l2[f]);
-        out[6 + f] = s[f] + c[f];
-    }
-    out[11] = bad;
+    sum_final(part, nblocks, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -1002,7 +955,7 @@ template <typename real>
 void Launch<real>::diag_partials(const JetDev<real> *jets, int jet, double *partials, int nblocks,
                                  cudaStream_t st)
 {
-    k_diag_partials<real><<<nblocks, BLOCK, 0, st>>>(jets, jet, partials);
+    k_diag_partials<real><<<nblocks, SUM_BLOCK, 0, st>>>(jets, jet, partials);
 }
 
 template <typename real>
@@ -1023,7 +976,7 @@ void Launch<real>::probe(const JetDev<real> *jets, const int *cell, const double
 
 void launch_diag_final(const double *partials, int nblocks, double *out, cudaStream_t st)
 {
-    k_diag_final<<<1, 32, 0, st>>>(partials, nblocks, out);
+    k_diag_final<<<1, SUM_FINAL_THREADS, 0, st>>>(partials, nblocks, out);
 }
 
 void launch_step_advance(long long *level, cudaStream_t st) { k_step_advance<<<1, 1, 0, st>>>(level); }

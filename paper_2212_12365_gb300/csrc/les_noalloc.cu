@@ -9,106 +9,46 @@
 // get the sums back in their own output buffer; this entry point allocates
 // nothing (no cudaMalloc, cudaFree or allocating library call).
 //
-// Its only scratch is the file-scope array g_partials below: one slot of
-// NA_NPART doubles per reduction block, at most NA_MAX_BLOCKS blocks.  Every
-// GPU that loads the library holds it (557 KB) until the process exits.
+// Its only scratch is the file-scope array g_partials below: SUM_PART doubles
+// per reduction block, at most SUM_MAX_BLOCKS blocks.  Every GPU that loads
+// the library holds it (83 KB) until the process exits.
 #include <cstdio>
 #include <mutex>
 
 #include "les_internal.cuh"
+#include "les_sums.cuh"
 
 namespace {
 
-constexpr int NA_BLOCK = 256;                      // threads per reduction block
-constexpr long long NA_POINTS_PER_BLOCK = 65536;   // points summed by one block
-constexpr int NA_MAX_BLOCKS = LES_NOALLOC_MAX_POINTS / 65536;
-constexpr int NA_NPART = 17;                       // partial results per block
-static_assert((long long)NA_MAX_BLOCKS * NA_POINTS_PER_BLOCK == LES_NOALLOC_MAX_POINTS,
-              "scratch size and the documented limit must agree");
+using namespace les;
 
-// Per-block partials: [0] max|RHS_rho|, [1..5] sum RHS_f^2, [6..10] Neumaier
-// sums of Qhat_f, [11..15] their compensations, [16] non-finite count.  Every
-// call overwrites the slots of the blocks it launches; nothing needs clearing.
-static __device__ __align__(256) double g_partials[NA_MAX_BLOCKS * NA_NPART];
+// Partials of the reduction blocks; every call overwrites what it reads.
+static __device__ __align__(256) double g_partials[SUM_MAX_BLOCKS * SUM_PART];
 
-__device__ __forceinline__ void na_neumaier(double &s, double &c, double v)
-{
-    double t = s + v;
-    if (fabs(s) >= fabs(v)) c += (s - t) + v;
-    else c += (v - t) + s;
-    s = t;
-}
-
-// Block b sums points [b*NA_POINTS_PER_BLOCK, (b+1)*NA_POINTS_PER_BLOCK) in a
-// fixed order (thread stride, then a shared-memory tree), so the result
+// Points are strided over the whole grid in a fixed order, so the result
 // depends only on the inputs and npoints.
-__global__ void __launch_bounds__(NA_BLOCK) k_na_partials(const double *__restrict__ qhat,
-                                                          const double *__restrict__ rhs,
-                                                          long long npoints, double *part)
+__global__ void __launch_bounds__(SUM_BLOCK, 4) k_na_partials(const double *__restrict__ qhat,
+                                                              const double *__restrict__ rhs,
+                                                              long long npoints, double *part)
 {
-    __shared__ double sh[NA_NPART][NA_BLOCK];
-    const long long p0 = (long long)blockIdx.x * NA_POINTS_PER_BLOCK;
-    long long p1 = p0 + NA_POINTS_PER_BLOCK;
-    if (p1 > npoints) p1 = npoints;
-    double mx = 0.0, bad = 0.0, l2[5] = {0, 0, 0, 0, 0}, s[5] = {0, 0, 0, 0, 0},
-           c[5] = {0, 0, 0, 0, 0};
-    for (long long p = p0 + threadIdx.x; p < p1; p += NA_BLOCK) {
-        for (int f = 0; f < 5; ++f) {
-            double r = rhs[f * npoints + p];
-            double v = qhat[f * npoints + p];
-            if (!isfinite(r) || !isfinite(v)) bad += 1.0;
-            l2[f] += r * r;
-            na_neumaier(s[f], c[f], v);
-        }
-        mx = fmax(mx, fabs(rhs[p]));
-    }
-    sh[0][threadIdx.x] = mx;
-    for (int f = 0; f < 5; ++f) {
-        sh[1 + f][threadIdx.x] = l2[f];
-        sh[6 + f][threadIdx.x] = s[f];
-        sh[11 + f][threadIdx.x] = c[f];
-    }
-    sh[16][threadIdx.x] = bad;
-    __syncthreads();
-    for (int st = NA_BLOCK / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            const int o = threadIdx.x + st;
-            sh[0][threadIdx.x] = fmax(sh[0][threadIdx.x], sh[0][o]);
-            for (int f = 0; f < 5; ++f) {
-                sh[1 + f][threadIdx.x] += sh[1 + f][o];
-                double a = sh[6 + f][threadIdx.x], ca = sh[11 + f][threadIdx.x];
-                na_neumaier(a, ca, sh[6 + f][o]);
-                sh[6 + f][threadIdx.x] = a;
-                sh[11 + f][threadIdx.x] = ca + sh[11 + f][o];
-            }
-            sh[16][threadIdx.x] += sh[16][o];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < NA_NPART) part[blockIdx.x * NA_NPART + threadIdx.x] = sh[threadIdx.x][0];
+    const long long stride = (long long)gridDim.x * SUM_BLOCK;
+    const long long p0 = blockIdx.x * (long long)SUM_BLOCK + threadIdx.x;
+    sum_block((npoints + stride - 1) / stride,
+              [&](long long t, double q[5], double r[5]) {
+                  const long long p = p0 + t * stride;
+#pragma unroll
+                  for (int f = 0; f < 5; ++f) {
+                      q[f] = p < npoints ? __ldcs(qhat + f * npoints + p) : 0.0;
+                      r[f] = p < npoints ? __ldcs(rhs + f * npoints + p) : 0.0;
+                  }
+              },
+              part);
 }
 
-__global__ void k_na_final(const double *__restrict__ part, int nblocks, double *out)
+__global__ void __launch_bounds__(SUM_FINAL_THREADS) k_na_final(const double *__restrict__ part, int nblocks,
+                                                                double *out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double mx = 0.0, bad = 0.0, l2[5] = {0, 0, 0, 0, 0}, s[5] = {0, 0, 0, 0, 0},
-           c[5] = {0, 0, 0, 0, 0};
-    for (int b = 0; b < nblocks; ++b) {
-        const double *P = part + (long long)b * NA_NPART;
-        mx = fmax(mx, P[0]);
-        for (int f = 0; f < 5; ++f) {
-            l2[f] += P[1 + f];
-            na_neumaier(s[f], c[f], P[6 + f]);
-            c[f] += P[11 + f];
-        }
-        bad += P[16];
-    }
-    out[0] = mx;
-    for (int f = 0; f < 5; ++f) {
-        out[1 + f] = sqrt(l2[f]);
-        out[6 + f] = s[f] + c[f];
-    }
-    out[11] = bad;
+    sum_final(part, nblocks, out);
 }
 
 // Device address of g_partials per device.  In host code the name
@@ -146,10 +86,10 @@ extern "C" int les_diag_sums_noalloc(const double *qhat, const double *rhs, int6
         }
         part = g_partials_addr[dev];
     }
-    const int nblocks = (int)((npoints + NA_POINTS_PER_BLOCK - 1) / NA_POINTS_PER_BLOCK);
+    const int nblocks = sum_blocks(npoints);
     cudaStream_t st = (cudaStream_t)stream;
-    k_na_partials<<<nblocks, NA_BLOCK, 0, st>>>(qhat, rhs, (long long)npoints, part);
-    k_na_final<<<1, 32, 0, st>>>(part, nblocks, out);
+    k_na_partials<<<nblocks, SUM_BLOCK, 0, st>>>(qhat, rhs, (long long)npoints, part);
+    k_na_final<<<1, SUM_FINAL_THREADS, 0, st>>>(part, nblocks, out);
     if (cudaGetLastError() != cudaSuccess) return LES_ERR_CUDA;
     return LES_OK;
 }
