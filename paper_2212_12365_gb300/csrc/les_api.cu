@@ -30,6 +30,7 @@ struct JetHost {
     les_params prm;
     bool product;                      // Cartesian-product grid (probe support)
     std::vector<double> ax[3];         // 1-D coordinates of a product grid
+    bool diag;                         // product grid with diagonal metrics and positive spacings
     size_t off;                        // byte offset of this jet's region
     size_t bytes;                      // size of this jet's region
     // device pointers (typed as bytes; the element type follows the precision)
@@ -37,12 +38,15 @@ struct JetHost {
     double *jinv64, *inflow_ut;
     float4 *h1[3];                     // FP32: 1-D spacings of a product grid (separable form)
     float4 *mp;                        // FP32 general form: paired static records (5 float4 / row pair)
-    int nblk_pt, nblk_bc[3];
+    double *ptab[3];                   // FP64: spacing tables of the product-grid stage
+    int nblk_pt, nblk_bc[3], nblk_prod;
 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 constexpr int DIAG_BLOCKS = SUM_MAX_BLOCKS; // blocks of the diagnostics reduction (scratch size)
+
+constexpr int MAP_FAMS = 6; // block maps of a handle
 
 } // namespace
 
@@ -63,7 +67,9 @@ struct les_handle {
     void *d_jets = nullptr;     // JetDev<real>[njets]
     int *d_maps = nullptr;      // block-start tables
     BlockMap pt{}, bcm[3]{};
+    BlockMap ptg{}, ptp{};             // FP64 stage: the jets of the general and of the product form
     std::vector<BlockMap> pt1, bc1[3]; // single-jet maps
+    std::vector<BlockMap> ptg1, ptp1;
     double *d_dt = nullptr;
     long long *d_level = nullptr;
     unsigned long long *d_dtbits = nullptr;
@@ -246,6 +252,7 @@ static void plan_jet(const les_grid_desc *g, int prec, JetHost &J)
     size_t o_inr = take((size_t)g->nj * g->nk * 8);
     size_t o_h1 = prec == LES_FP32 ? take((size_t)(g->ni + g->nj + g->nk) * 16) : 0;
     const bool packed = g->precision == LES_FP32; // general FP32 form only
+    size_t o_pt = prec == LES_FP64 ? take((size_t)(g->ni + g->nj + g->nk) * PROD_TABS * 8) : 0;
     size_t o_mp = packed ? take((size_t)g->nk * ((g->nj + 1) / 2) * J.pitch * 80) : 0;
     J.bytes = off;
     // store offsets relative to the jet region in the pointers for now
@@ -263,6 +270,9 @@ static void plan_jet(const les_grid_desc *g, int prec, JetHost &J)
     J.h1[1] = prec == LES_FP32 ? (float4 *)(o_h1 + (size_t)g->ni * 16) : nullptr;
     J.h1[2] = prec == LES_FP32 ? (float4 *)(o_h1 + (size_t)(g->ni + g->nj) * 16) : nullptr;
     J.mp = packed ? (float4 *)o_mp : nullptr;
+    J.ptab[0] = prec == LES_FP64 ? (double *)o_pt : nullptr;
+    J.ptab[1] = prec == LES_FP64 ? (double *)(o_pt + (size_t)g->ni * PROD_TABS * 8) : nullptr;
+    J.ptab[2] = prec == LES_FP64 ? (double *)(o_pt + (size_t)(g->ni + g->nj) * PROD_TABS * 8) : nullptr;
 }
 
 // Storage precision of a descriptor's precision code.
@@ -282,7 +292,7 @@ static GlobalPlan plan_global(int njets, size_t jetdev_bytes, int nblk_diag, lon
         return o;
     };
     P.o_jets = take(jetdev_bytes * njets);
-    P.o_maps = take(sizeof(int) * 4 * (njets + 1) + sizeof(int) * 8 * njets);
+    P.o_maps = take(sizeof(int) * MAP_FAMS * (3 * (size_t)njets + 1));
     P.o_dt = take(sizeof(double) * njets);
     P.o_level = take(sizeof(long long));
     P.o_bits = take(sizeof(unsigned long long) * njets);
@@ -332,6 +342,7 @@ template <typename real> static void fill_jetdev(const les_handle *h, const JetH
     D.hflux = (real *)J.hflux;
     D.rhs = (real *)J.rhs;
     D.inflow_ut = J.inflow_ut;
+    for (int a = 0; a < 3; ++a) D.ptab[a] = J.ptab[a];
     D.oob = h->d_oob;
     const les_params &p = J.prm;
     D.gamma = p.gamma;
@@ -429,6 +440,26 @@ template <typename real> static int setup_jet(les_handle *h, JetHost &J, const l
         for (int i = 0; i < J.n[0]; ++i) J.ax[0].push_back(g->x[i]);
         for (int j = 0; j < J.n[1]; ++j) J.ax[1].push_back(g->y[(size_t)j * J.n[0]]);
         for (int k = 0; k < J.n[2]; ++k) J.ax[2].push_back(g->z[(size_t)k * J.n[0] * J.n[1]]);
+    }
+    // The stage forms with diagonal metrics take a product grid whose period
+    // shifts run along their own axes and whose spacings are all positive (the
+    // spectral radius (|u| + c)/h of an axis needs h > 0; two descending axes
+    // would give a positive volume with negative spacings).
+    J.diag = J.product;
+    for (int a = 0; a < 3; ++a)
+        for (int c = 0; c < 3; ++c)
+            if (J.per[a] && c != a && J.shift[3 * a + c] != 0.0) J.diag = false;
+    if (J.diag && h->prec == LES_FP64) {
+        launch_prod_tables(dx, dy, dz, J.n, J.per, J.shift, J.ptab, h->st);
+        CK(cudaGetLastError());
+        for (int a = 0; a < 3; ++a) {
+            std::vector<double> ha(J.n[a]);
+            CK(cudaMemcpyAsync(ha.data(), J.ptab[a] + (size_t)PT_H * J.n[a], ha.size() * 8, cudaMemcpyDeviceToHost,
+                               h->st));
+            CK(cudaStreamSynchronize(h->st));
+            for (double v : ha)
+                if (!(v > 0.0)) J.diag = false;
+        }
     }
     return LES_OK;
 }
@@ -575,6 +606,7 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
         for (int a = 0; a < 3; ++a)
             for (int c = 0; c < 3; ++c) J.shift[3 * a + c] = g[j].period_shift[a][c];
         J.nblk_pt = (int)((J.npad + BLOCK - 1) / BLOCK);
+        J.nblk_prod = (int)((J.npad + PROD_BLOCK - 1) / PROD_BLOCK);
         for (int a = 0; a < 3; ++a) {
             if (J.per[a]) {
                 J.nblk_bc[a] = 0;
@@ -637,6 +669,8 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
         for (int a = 0; a < 3; ++a)
             if (J.h1[a]) J.h1[a] = (float4 *)(jb + (size_t)J.h1[a]);
         if (J.mp) J.mp = (float4 *)(jb + (size_t)J.mp);
+        for (int a = 0; a < 3; ++a)
+            if (J.ptab[a]) J.ptab[a] = (double *)(jb + (size_t)J.ptab[a]);
     }
     for (int j = 0; j < njets; ++j) {
         int rc = setup_jet<real>(h, h->J[j], &g[j]);
@@ -688,29 +722,29 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
         int rc = set_fused_tiling(h, 8, 32);
         if (rc) return bail(rc);
     }
-    // block maps: [pt | bc0 | bc1 | bc2] each njets+1, then per-jet pairs
-    std::vector<int> maps(4 * (njets + 1) + 8 * njets);
-    for (int fam = 0; fam < 4; ++fam) {
+    // block maps: [pt | bc0 | bc1 | bc2 | ptg | ptp] each njets+1, then per-jet pairs
+    std::vector<int> maps(MAP_FAMS * (njets + 1) + 2 * MAP_FAMS * njets);
+    BlockMap *all[MAP_FAMS] = {&h->pt, &h->bcm[0], &h->bcm[1], &h->bcm[2], &h->ptg, &h->ptp};
+    std::vector<BlockMap> *one[MAP_FAMS] = {&h->pt1, &h->bc1[0], &h->bc1[1], &h->bc1[2], &h->ptg1, &h->ptp1};
+    int *pj = maps.data() + MAP_FAMS * (njets + 1);
+    for (int fam = 0; fam < MAP_FAMS; ++fam) {
         int acc = 0;
+        one[fam]->resize(njets);
         for (int j = 0; j < njets; ++j) {
+            const JetHost &J = h->J[j];
+            const int nb = fam == 0 ? J.nblk_pt
+                           : fam < 4 ? J.nblk_bc[fam - 1]
+                           : fam == 4 ? (J.diag ? 0 : J.nblk_pt)
+                                      : (J.diag ? J.nblk_prod : 0);
             maps[fam * (njets + 1) + j] = acc;
-            acc += fam == 0 ? h->J[j].nblk_pt : h->J[j].nblk_bc[fam - 1];
+            acc += nb;
+            const int o = 2 * (MAP_FAMS * j + fam);
+            pj[o] = 0;
+            pj[o + 1] = nb;
+            (*one[fam])[j] = BlockMap{h->d_maps + MAP_FAMS * (njets + 1) + o, 1, nb};
         }
         maps[fam * (njets + 1) + njets] = acc;
-        BlockMap bm{h->d_maps + fam * (njets + 1), njets, acc};
-        if (fam == 0) h->pt = bm; else h->bcm[fam - 1] = bm;
-    }
-    int *pj = maps.data() + 4 * (njets + 1);
-    h->pt1.resize(njets);
-    for (int a = 0; a < 3; ++a) h->bc1[a].resize(njets);
-    for (int j = 0; j < njets; ++j) {
-        for (int fam = 0; fam < 4; ++fam) {
-            int nb = fam == 0 ? h->J[j].nblk_pt : h->J[j].nblk_bc[fam - 1];
-            pj[8 * j + 2 * fam] = 0;
-            pj[8 * j + 2 * fam + 1] = nb;
-            BlockMap bm{h->d_maps + 4 * (njets + 1) + 8 * j + 2 * fam, 1, nb};
-            if (fam == 0) h->pt1[j] = bm; else h->bc1[fam - 1][j] = bm;
-        }
+        *all[fam] = BlockMap{h->d_maps + fam * (njets + 1), njets, acc};
     }
     CK(cudaMemcpyAsync(h->d_maps, maps.data(), maps.size() * sizeof(int), cudaMemcpyHostToDevice, h->st));
     CK(cudaMemsetAsync(h->d_level, 0, sizeof(long long), h->st));
@@ -779,19 +813,24 @@ extern "C" int les_create_batch(const les_grid_desc *g, const les_params *p, int
 
 static int grid_cap(les_handle *h, int total) { return std::max(1, std::min(total, h->nsm * 8)); }
 
-template <typename real>
-static int rhs_pass(les_handle *h, const BlockMap &pt, const JetDev<real> *jets, int src,
-                    int rhs_only, int dst, int stage)
+// One part (0 point, 1 gradients, 2 interfaces, 3 update) of the FP64 stage:
+// the jets of the general form (map g), then those of the product form (map
+// p); returns the number of launches.
+static int fp64_part(les_handle *h, const JetDev<double> *jets, const BlockMap &g, const BlockMap &p, int part, int src,
+                     int dst, int stage, int rhs_only, cudaStream_t st)
 {
-    // the four-kernel stage needs the FP64 interface tables
-    if (h->prec != LES_FP64) return fail(h, LES_ERR_STATE, "four-kernel stage on an FP32 handle");
-    int gp = grid_cap(h, pt.total);
-    Launch<real>::point(jets, pt, src, gp, h->st);
-    Launch<real>::grads(jets, pt, gp, h->st);
-    Launch<real>::iface(jets, pt, gp, h->st);
-    Launch<real>::update(jets, pt, dst, stage, h->d_dt, rhs_only, gp, h->st);
-    CK(cudaGetLastError());
-    return LES_OK;
+    if (g.total > 0) {
+        const int gp = grid_cap(h, g.total);
+        switch (part) {
+        case 0: Launch<double>::point(jets, g, src, gp, st); break;
+        case 1: Launch<double>::grads(jets, g, gp, st); break;
+        case 2: Launch<double>::iface(jets, g, gp, st); break;
+        default: Launch<double>::update(jets, g, dst, stage, h->d_dt, rhs_only, gp, st); break;
+        }
+    }
+    // one block per 64 points: the hardware balances them over the SMs
+    if (p.total > 0) launch_stage_prod(jets, p, part, src, dst, stage, h->d_dt, rhs_only, p.total, st);
+    return (g.total > 0) + (p.total > 0);
 }
 
 template <typename real>
@@ -847,7 +886,6 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
     launch_step_advance(h->d_level, st);
     T.end();
     h->launches_per_step++;
-    int gp = grid_cap(h, h->pt.total);
     for (int s = 0; s < 5; ++s) {
         if (h->prec == LES_FP32) {
             // fused single-pass stage: counted as the interface kernel kind
@@ -871,19 +909,12 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
             }
             continue;
         }
-        T.begin(LES_KERNEL_POINT);
-        Launch<real>::point(jets, h->pt, src_of[s], gp, st);
-        T.end();
-        T.begin(LES_KERNEL_GRADS);
-        Launch<real>::grads(jets, h->pt, gp, st);
-        T.end();
-        T.begin(LES_KERNEL_IFACE);
-        Launch<real>::iface(jets, h->pt, gp, st);
-        T.end();
-        T.begin(LES_KERNEL_UPDATE);
-        Launch<real>::update(jets, h->pt, dst_of[s], s, h->d_dt, 0, gp, st);
-        T.end();
-        h->launches_per_step += 4;
+        for (int part = 0; part < 4; ++part) {
+            T.begin(LES_KERNEL_POINT + part);
+            h->launches_per_step += fp64_part(h, (const JetDev<double> *)h->d_jets, h->ptg, h->ptp, part, src_of[s],
+                                              dst_of[s], s, 0, st);
+            T.end();
+        }
         for (int oi = 0; oi < 3; ++oi) {
             int a = order[oi];
             if (a == 1 && h->centerline) {
@@ -1093,8 +1124,10 @@ template <typename real> static int residual_of_jet(les_handle *h, int jet)
         CK(cudaGetLastError());
         return LES_OK;
     }
-    const JetDev<real> *one = (const JetDev<real> *)h->d_jets + jet;
-    return rhs_pass<real>(h, h->pt1[jet], one, 0, 1, 0, 0);
+    for (int part = 0; part < 4; ++part)
+        fp64_part(h, (const JetDev<double> *)h->d_jets + jet, h->ptg1[jet], h->ptp1[jet], part, 0, 0, 0, 1, h->st);
+    CK(cudaGetLastError());
+    return LES_OK;
 }
 
 // Autotuner of the fused stage: time (tile height, k-chunk) candidates with
@@ -1378,7 +1411,7 @@ extern "C" const char *les_describe(les_handle *h)
     static thread_local std::string d;
     d = std::string(h->prec == LES_FP64 ? "fp64" : "fp32") + " jets=" + std::to_string(h->njets) +
         " device_bytes=" + std::to_string(h->bytes) + " stage=" +
-        (h->prec == LES_FP64 ? std::string("point+grads+iface+update")
+        (h->prec == LES_FP64 ? std::string("point+grads+iface+update") + (h->ptg.total == 0 ? " (product)" : h->ptp.total > 0 ? " (general, product)" : " (general)")
                              : std::string(h->sep ? "fused separable " : "fused ") + (h->tuned ? h->tune_note : "ty=" + std::to_string(h->fused_ty) + " (untuned)")) +
         " launches_per_step=" + std::to_string(h->launches_per_step);
     return d.c_str();

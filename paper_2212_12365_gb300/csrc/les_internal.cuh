@@ -57,6 +57,11 @@ constexpr int G_NU = 15;      // + a
 constexpr int NHF = 15;       // interface fluxes H_a at [5a + f], interface L + e_a/2
 
 constexpr int BLOCK = 256;    // threads per block of the point / face kernels
+constexpr int PROD_BLOCK = 64; // threads per block of the product-grid FP64 stage (les_stage_prod.cu)
+// Spacing tables of the product-grid FP64 stage, per axis [table][index]: h =
+// d x_a / d xi^a; 1/h; 1/(4h); 1/(6h); hb = the mean of h over the interface
+// to the next point; 1/hb; 4/(3 hb).
+enum { PT_H = 0, PT_RH, PT_RH4, PT_RH6, PT_HB, PT_RHB, PT_RHB43, PROD_TABS };
 constexpr int DBG_RHS = 100;  // debug export codes beside the LES_FIELD_* values
 constexpr int DBG_MET0 = 200;
 
@@ -77,6 +82,7 @@ struct JetDev {
     real *grad;        // NGRAD fields (scratch)
     real *hflux;       // NHF fields (scratch): interface fluxes
     real *rhs;         // NF fields (residual for diagnostics / debug)
+    const double *ptab[3];   // FP64 product grids: PROD_TABS tables of n[a] entries per axis
     const double *inflow_ut; // nj*nk: inflow profile u~(r) of the i = 0 face points (host tanh)
     // flow parameters (jet units)
     double gamma, Pr, Pr_sgs, Re, mach, TR, theta, noise_amp, k2, k4, suth_S;
@@ -296,6 +302,15 @@ void launch_pack_pairs(const float *met, long long fs, int pitch, int nj, int nk
 // coordinates (FP64 derivative stencils of the metric computation).
 void launch_sep_metrics(const double *x, const double *y, const double *z, const int n[3], const int per[3],
                         const double shift[9], float4 *h1x, float4 *h1y, float4 *h1z, cudaStream_t st);
+
+// FP64 stage on Cartesian-product grids (les_stage_prod.cu): part 0 point, 1
+// gradients, 2 interfaces, 3 update; bm maps blocks of PROD_BLOCK points.
+void launch_stage_prod(const JetDev<double> *jets, BlockMap bm, int part, int src, int dst, int stage,
+                       const double *dt, int rhs_only, int grid, cudaStream_t st);
+// Its spacing tables, from device coordinates, and the three h tables' place
+// in the result for the caller's check.
+void launch_prod_tables(const double *x, const double *y, const double *z, const int n[3], const int per[3],
+                        const double shift[9], double *const tab[3], cudaStream_t st);
 
 // Kernel launchers (les_kernels.cu, les_stage.cu), all asynchronous on `st`.
 template <typename real> struct Launch {

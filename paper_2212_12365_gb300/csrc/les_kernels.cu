@@ -162,6 +162,45 @@ void launch_sep_metrics(const double *x, const double *y, const double *z, const
     k_sep_metrics<<<(tot + BLOCK - 1) / BLOCK, BLOCK, 0, st>>>(G, h1x, h1y, h1z);
 }
 
+// Spacing tables of the product-grid FP64 stage (PROD_TABS per axis).
+__global__ void __launch_bounds__(BLOCK) k_prod_tables(CoordGrid G, double *t0, double *t1, double *t2)
+{
+    const int tot = G.n[0] + G.n[1] + G.n[2];
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += gridDim.x * blockDim.x) {
+        const int a = t < G.n[0] ? 0 : (t < G.n[0] + G.n[1] ? 1 : 2);
+        const int n = G.n[a], i = a == 0 ? t : (a == 1 ? t - G.n[0] : t - G.n[0] - G.n[1]);
+        int q[3] = {0, 0, 0};
+        q[a] = i;
+        const double h = dcoord(G, a, a, q);
+        q[a] = i + 1 < n ? i + 1 : (G.per[a] ? 0 : i);
+        const double hb = 0.5 * (h + dcoord(G, a, a, q));
+        double *o = (a == 0 ? t0 : (a == 1 ? t1 : t2)) + i;
+        o[PT_H * n] = h;
+        o[PT_RH * n] = 1.0 / h;
+        o[PT_RH4 * n] = 0.25 / h;
+        o[PT_RH6 * n] = 1.0 / (6.0 * h);
+        o[PT_HB * n] = hb;
+        o[PT_RHB * n] = 1.0 / hb;
+        o[PT_RHB43 * n] = 4.0 / (3.0 * hb);
+    }
+}
+
+void launch_prod_tables(const double *x, const double *y, const double *z, const int n[3], const int per[3],
+                        const double shift[9], double *const tab[3], cudaStream_t st)
+{
+    CoordGrid G;
+    G.X[0] = x;
+    G.X[1] = y;
+    G.X[2] = z;
+    for (int a = 0; a < 3; ++a) {
+        G.n[a] = n[a];
+        G.per[a] = per[a];
+    }
+    for (int t = 0; t < 9; ++t) G.shift[t] = shift[t];
+    const int tot = n[0] + n[1] + n[2];
+    k_prod_tables<<<(tot + BLOCK - 1) / BLOCK, BLOCK, 0, st>>>(G, tab[0], tab[1], tab[2]);
+}
+
 // Static per-point fields derived from the metrics (FP64): J = 1/J^-1; per
 // axis a the interface average of J^-1 towards the +a neighbour, its
 // reciprocal, and the norm of metric row a.
