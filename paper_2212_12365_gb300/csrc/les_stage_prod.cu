@@ -14,8 +14,9 @@
 // with F the Cartesian point fluxes (nine products, rho u_i u_j is symmetric),
 // and the update multiplies each flux difference by S_a / 2 once.
 // FP64 instructions per point: point 65, gradients 63, interfaces 3 x 56,
-// update 36 = 332.  Measured: four steps of the 384x256x144 jet 331.6 -> 218.0 ms,
-// ten of the 48x32x32 jet 9.84 -> 7.74 ms.
+// update 36 = 332.  Measured on the 384x256x144 jet, us per launch, general ->
+// this form: point 2740 -> 1717, gradients 2710 -> 1682, interfaces 8385 ->
+// 4202 (FP64 pipe 85-88 % busy in each), update 952 -> 924.
 // Tangential derivatives reach the interface as c_ai = (1/2) du_a/dx_i and the
 // divergence as the third s_a = (1/3) sum_{i != a} du_i/dx_i of each point, so
 // that the sums over the two points need no factor.
@@ -152,7 +153,19 @@ __device__ __forceinline__ void axis_diff(const JetDev<double> &J, const Pt &pt,
     for (int i = 0; i < 3; ++i) {
         const double *F = P + (R_U + i) * fs;
         d[i] = F[o2] - F[o1];
-        if (end) d[i] = (double)t * fma(-3.0, F[pt.lp], fma(3.0, F[o1], -d[i])); // t (4 f1 - 3 f0 - f2)
+    }
+    // a vote, so that this stays a branch: as predicated instructions the
+    // one-sided form cost every point a third of the pass (93 instead of 63
+    // FP64 instructions, 2444 instead of 1682 us on the 384x256x144 jet)
+    if (__ballot_sync(__activemask(), end)) {
+        if (end) {
+            const double td = t > 0 ? 1.0 : -1.0;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const double *F = P + (R_U + i) * fs;
+                d[i] = td * fma(-3.0, F[pt.lp], fma(3.0, F[o1], -d[i])); // t (4 f1 - 3 f0 - f2)
+            }
+        }
     }
     const double *F = P + R_P * fs;
     const double p0 = F[pt.lp], p1 = F[o1], p2 = F[o2];
