@@ -39,14 +39,14 @@ struct JetHost {
     float4 *h1[3];                     // FP32: 1-D spacings of a product grid (separable form)
     float4 *mp;                        // FP32 general form: paired static records (5 float4 / row pair)
     double *ptab[3];                   // FP64: spacing tables of the product-grid stage
-    int nblk_pt, nblk_bc[3], nblk_prod;
+    int nblk_pt, nblk_bc, nblk_prod;
 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 constexpr int DIAG_BLOCKS = SUM_MAX_BLOCKS; // blocks of the diagnostics reduction (scratch size)
 
-constexpr int MAP_FAMS = 6; // block maps of a handle
+constexpr int MAP_FAMS = 4; // block maps of a handle
 
 } // namespace
 
@@ -66,9 +66,9 @@ struct les_handle {
     std::vector<JetHost> J;
     void *d_jets = nullptr;     // JetDev<real>[njets]
     int *d_maps = nullptr;      // block-start tables
-    BlockMap pt{}, bcm[3]{};
+    BlockMap pt{}, bcm{};
     BlockMap ptg{}, ptp{};             // FP64 stage: the jets of the general and of the product form
-    std::vector<BlockMap> pt1, bc1[3]; // single-jet maps
+    std::vector<BlockMap> pt1, bc1;    // single-jet maps
     std::vector<BlockMap> ptg1, ptp1;
     double *d_dt = nullptr;
     long long *d_level = nullptr;
@@ -607,14 +607,7 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
             for (int c = 0; c < 3; ++c) J.shift[3 * a + c] = g[j].period_shift[a][c];
         J.nblk_pt = (int)((J.npad + BLOCK - 1) / BLOCK);
         J.nblk_prod = (int)((J.npad + PROD_BLOCK - 1) / PROD_BLOCK);
-        for (int a = 0; a < 3; ++a) {
-            if (J.per[a]) {
-                J.nblk_bc[a] = 0;
-                continue;
-            }
-            long long nface = (long long)J.n[(a + 1) % 3] * J.n[(a + 2) % 3];
-            J.nblk_bc[a] = (int)((2 * nface + BLOCK - 1) / BLOCK);
-        }
+        J.nblk_bc = bc_blocks(J.n, J.per);
         J.off = jets_bytes;
         jets_bytes += align_up(J.bytes, 256);
         maxN = std::max(maxN, J.N);
@@ -722,10 +715,10 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
         int rc = set_fused_tiling(h, 8, 32);
         if (rc) return bail(rc);
     }
-    // block maps: [pt | bc0 | bc1 | bc2 | ptg | ptp] each njets+1, then per-jet pairs
+    // block maps: [pt | bc | ptg | ptp] each njets+1, then per-jet pairs
     std::vector<int> maps(MAP_FAMS * (njets + 1) + 2 * MAP_FAMS * njets);
-    BlockMap *all[MAP_FAMS] = {&h->pt, &h->bcm[0], &h->bcm[1], &h->bcm[2], &h->ptg, &h->ptp};
-    std::vector<BlockMap> *one[MAP_FAMS] = {&h->pt1, &h->bc1[0], &h->bc1[1], &h->bc1[2], &h->ptg1, &h->ptp1};
+    BlockMap *all[MAP_FAMS] = {&h->pt, &h->bcm, &h->ptg, &h->ptp};
+    std::vector<BlockMap> *one[MAP_FAMS] = {&h->pt1, &h->bc1, &h->ptg1, &h->ptp1};
     int *pj = maps.data() + MAP_FAMS * (njets + 1);
     for (int fam = 0; fam < MAP_FAMS; ++fam) {
         int acc = 0;
@@ -733,8 +726,8 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
         for (int j = 0; j < njets; ++j) {
             const JetHost &J = h->J[j];
             const int nb = fam == 0 ? J.nblk_pt
-                           : fam < 4 ? J.nblk_bc[fam - 1]
-                           : fam == 4 ? (J.diag ? 0 : J.nblk_pt)
+                           : fam == 1 ? J.nblk_bc
+                           : fam == 2 ? (J.diag ? 0 : J.nblk_pt)
                                       : (J.diag ? J.nblk_prod : 0);
             maps[fam * (njets + 1) + j] = acc;
             acc += nb;
@@ -833,23 +826,14 @@ static int fp64_part(les_handle *h, const JetDev<double> *jets, const BlockMap &
     return (g.total > 0) + (p.total > 0);
 }
 
+// Boundary conditions of the current level on the jets of the map; returns the
+// number of launches.
 template <typename real>
-static int bc_pass(les_handle *h, const BlockMap bcm[3], const JetDev<real> *jets, int dst,
-                   cudaStream_t st)
+static int bc_pass(les_handle *h, const BlockMap &bm, const JetDev<real> *jets, int dst, cudaStream_t st)
 {
-    static const int order[3] = {1, 2, 0};
-    for (int oi = 0; oi < 3; ++oi) {
-        int a = order[oi];
-        if (a == 1 && h->centerline) {
-            launch_centerline<real>(jets, bcm[1].njets, h->max_ni, dst, st);
-            h->launches_per_step++;
-        }
-        if (bcm[a].total == 0) continue;
-        Launch<real>::bc(jets, bcm[a], a, dst, h->d_level, grid_cap(h, bcm[a].total), st);
-        h->launches_per_step++;
-    }
-    CK(cudaGetLastError());
-    return LES_OK;
+    if (h->centerline) launch_centerline<real>(jets, bm.njets, h->max_ni, dst, st);
+    Launch<real>::bc(jets, bm, dst, h->d_level, st);
+    return (h->centerline ? 1 : 0) + (bm.total > 0 ? 1 : 0);
 }
 
 // Optional per-launch event timing (les_profile_step); inactive during capture.
@@ -880,7 +864,6 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
     const JetDev<real> *jets = (const JetDev<real> *)h->d_jets;
     static const int src_of[5] = {0, 1, 2, 1, 2};
     static const int dst_of[5] = {1, 2, 1, 2, 0};
-    static const int order[3] = {1, 2, 0};
     h->launches_per_step = 0;
     T.begin(LES_KERNEL_OTHER);
     launch_step_advance(h->d_level, st);
@@ -893,19 +876,10 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
             fused_launch(h, -1, src_of[s], dst_of[s], s, 0, st);
             T.end();
             h->launches_per_step += 1;
-            for (int oi = 0; oi < 3; ++oi) {
-                int a = order[oi];
-                if (a == 1 && h->centerline) {
-                    T.begin(LES_KERNEL_BC);
-                    launch_centerline<real>(jets, h->njets, h->max_ni, dst_of[s], st);
-                    T.end();
-                    h->launches_per_step++;
-                }
-                if (h->bcm[a].total == 0) continue;
+            if (h->bcm.total > 0) { // none on a fully periodic grid
                 T.begin(LES_KERNEL_BC);
-                Launch<real>::bc(jets, h->bcm[a], a, dst_of[s], h->d_level, grid_cap(h, h->bcm[a].total), st);
+                h->launches_per_step += bc_pass<real>(h, h->bcm, jets, dst_of[s], st);
                 T.end();
-                h->launches_per_step++;
             }
             continue;
         }
@@ -915,19 +889,10 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
                                               dst_of[s], s, 0, st);
             T.end();
         }
-        for (int oi = 0; oi < 3; ++oi) {
-            int a = order[oi];
-            if (a == 1 && h->centerline) {
-                T.begin(LES_KERNEL_BC);
-                launch_centerline<real>(jets, h->njets, h->max_ni, dst_of[s], st);
-                T.end();
-                h->launches_per_step++;
-            }
-            if (h->bcm[a].total == 0) continue;
+        if (h->bcm.total > 0) { // none on a fully periodic grid
             T.begin(LES_KERNEL_BC);
-            Launch<real>::bc(jets, h->bcm[a], a, dst_of[s], h->d_level, grid_cap(h, h->bcm[a].total), st);
+            h->launches_per_step += bc_pass<real>(h, h->bcm, jets, dst_of[s], st);
             T.end();
-            h->launches_per_step++;
         }
     }
     if (h->probe_npts > 0) {
@@ -1037,11 +1002,8 @@ template <typename real> static int set_state_impl(les_handle *h, int jet, const
     CK(cudaGetLastError());
     // boundary conditions of the current level on this jet (faces y, z, x)
     const JetDev<real> *one = jets + jet;
-    BlockMap b1[3] = {h->bc1[0][jet], h->bc1[1][jet], h->bc1[2][jet]};
-    int64_t saved = h->launches_per_step;
-    int rc = bc_pass<real>(h, b1, one, 0, h->st);
-    h->launches_per_step = saved;
-    if (rc) return rc;
+    bc_pass<real>(h, h->bc1[jet], one, 0, h->st);
+    CK(cudaGetLastError());
     if (h->dt[jet] == 0.0) {
         BlockMap p1 = h->pt1[jet];
         Launch<real>::point(one, p1, 0, grid_cap(h, p1.total), h->st);

@@ -40,6 +40,13 @@ __device__ __forceinline__ double rcp64_1(double b)
     const double r = rcp_seed64(b);
     return fma(r, fma(-b, r, 1.0), r);
 }
+// x^-1/2, x positive and normal
+__device__ __forceinline__ double rsqrt64(double x)
+{
+    const double y = rsqrt_seed64(x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y, e * fma(0.375, e, 0.5), y);
+}
 // x^1/2, x >= 0; 0 below the normal range
 __device__ __forceinline__ double sqrt64_scaled(double x, int twice)
 {

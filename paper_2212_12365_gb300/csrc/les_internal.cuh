@@ -326,8 +326,7 @@ template <typename real> struct Launch {
     static void iface(const JetDev<real> *jets, BlockMap bm, int grid, cudaStream_t st);
     static void update(const JetDev<real> *jets, BlockMap bm, int dst, int stage,
                        const double *dt, int rhs_only, int grid, cudaStream_t st);
-    static void bc(const JetDev<real> *jets, BlockMap bm, int axis, int dst,
-                   const long long *level, int grid, cudaStream_t st);
+    static void bc(const JetDev<real> *jets, BlockMap bm, int dst, const long long *level, cudaStream_t st);
     static void set_state(const JetDev<real> *jets, int jet, const double *in, int kind,
                           long long npad, cudaStream_t st);
     static void get_state(const JetDev<real> *jets, int jet, double *out, int kind,
@@ -343,6 +342,9 @@ template <typename real> struct Launch {
                       int every, const long long *level, const long long *base, real *out,
                       int capacity, cudaStream_t st);
 };
+
+// Blocks of the boundary pass of one jet.
+int bc_blocks(const int n[3], const int per[3]);
 
 // Centerline faces (j- face of type LES_BC_CENTERLINE) of jets [0, njets):
 // the conserved variables of every axis point are the azimuthal mean of the
