@@ -87,16 +87,20 @@ struct les_handle {
     std::vector<double> dt;
     std::vector<char> has_state;
     cudaGraphExec_t gexec = nullptr;
-    // fused FP32 stage: work-list tables (all jets; and one per jet with item0 = 0)
-    FusedJet *d_fj = nullptr, *d_fj1 = nullptr;
-    std::vector<FusedJet> fj, fj1; // host copies of d_fj and d_fj1
-    std::vector<JetDev<float>> jd32; // host copy of the FP32 jet table
-    int fused_ty = 16;
-    int fused_balanced = 0; // 0: k-chunk items, 1: balanced ranges, 2: lockstep waves, then balanced ranges
-    int fused_items = 0, fused_tiles = 0;
-    int fused_cps[2] = {1, 1}; // resident CTAs per SM of the fused stage at tile height 8, 16
+    // fused FP32 stage: work lists of its two forms (general metrics; product
+    // grids), each over all jets (a jet has no items in the other form's list)
+    struct Form {
+        bool any = false;               // some jet takes this form
+        FusedJet *d_fj = nullptr, *d_fj1 = nullptr; // all jets; one per jet with item0 = 0
+        std::vector<FusedJet> fj, fj1;  // host copies
+        int ty = 16;
+        int balanced = 0;               // 0: k-chunk items, 1: balanced ranges, 2: lockstep waves, then balanced ranges
+        int items = 0, tiles = 0;
+        int cps[3] = {1, 1, 1};         // resident CTAs per SM at tile height 8, 16, 24
+        std::string note;
+    } form[2];
+    std::vector<JetDev<float>> jd32;    // host copy of the FP32 jet table
     bool tuned = false;
-    std::string tune_note;
     int64_t launches_per_step = 0;
     int64_t last_launches = 0;
     // probe
@@ -300,9 +304,9 @@ static GlobalPlan plan_global(int njets, size_t jetdev_bytes, int nblk_diag, lon
     P.o_diag = take(sizeof(double) * 16);
     P.o_pbase = take(sizeof(long long));
     P.o_stage = take(sizeof(double) * 5 * (size_t)maxN);
-    P.o_fj = take(sizeof(FusedJet) * 2 * njets);
+    P.o_fj = take(sizeof(FusedJet) * 4 * njets);
     P.o_oob = take(sizeof(unsigned long long));
-    P.o_tmap = take(sizeof(CUtensorMap) * 6 * njets);
+    P.o_tmap = take(sizeof(CUtensorMap) * 9 * njets);
     P.total = off;
     return P;
 }
@@ -387,19 +391,11 @@ template <typename real> static int setup_jet(les_handle *h, JetHost &J, const l
     CK(cudaGetLastError());
     Launch<real>::static_fields(met64, J.fs, J.pitch, J.n, J.per, h->prec == LES_FP64 ? 1 : 0, h->st);
     CK(cudaGetLastError());
-    if (h->sep) {
-        launch_sep_metrics(dx, dy, dz, J.n, J.per, J.shift, J.h1[0], J.h1[1], J.h1[2], h->st);
-        CK(cudaGetLastError());
-    }
     if (h->prec == LES_FP32) {
         Launch<real>::convert_metrics(met64, J.fs, (real *)J.met, J.fs, J.npad, h->st);
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(J.jinv64, met64 + MET_JINV * J.fs, (size_t)J.fs * 8,
                            cudaMemcpyDeviceToDevice, h->st));
-        if (J.mp) {
-            launch_pack_pairs((const float *)J.met, J.fs, J.pitch, J.n[1], J.n[2], J.mp, h->st);
-            CK(cudaGetLastError());
-        }
     }
     // inflow profile u~(r) = [1 + tanh((0.5 - r)/(2 theta))]/2 of the
     // inflow-face points, r = (y^2 + z^2)^1/2 (static: formed once here)
@@ -449,6 +445,19 @@ template <typename real> static int setup_jet(les_handle *h, JetHost &J, const l
     for (int a = 0; a < 3; ++a)
         for (int c = 0; c < 3; ++c)
             if (J.per[a] && c != a && J.shift[3 * a + c] != 0.0) J.diag = false;
+    if (J.product && h->prec == LES_FP32) {
+        launch_sep_metrics(dx, dy, dz, J.n, J.per, J.shift, J.h1[0], J.h1[1], J.h1[2], h->st);
+        CK(cudaGetLastError());
+        std::vector<float4> ha((size_t)J.n[0] + J.n[1] + J.n[2]); // the three tables are contiguous
+        CK(cudaMemcpyAsync(ha.data(), J.h1[0], ha.size() * sizeof(float4), cudaMemcpyDeviceToHost, h->st));
+        CK(cudaStreamSynchronize(h->st));
+        for (const float4 &v : ha)
+            if (!(v.x > 0.0f)) J.diag = false;
+    }
+    if (h->prec == LES_FP32 && !h->sep && !J.diag) {
+        launch_pack_pairs((const float *)J.met, J.fs, J.pitch, J.n[1], J.n[2], J.mp, h->st);
+        CK(cudaGetLastError());
+    }
     if (J.diag && h->prec == LES_FP64) {
         launch_prod_tables(dx, dy, dz, J.n, J.per, J.shift, J.ptab, h->st);
         CK(cudaGetLastError());
@@ -467,18 +476,25 @@ template <typename real> static int setup_jet(les_handle *h, JetHost &J, const l
 // Interior output range length of one axis.
 static int out_len(const JetHost &J, int a) { return J.per[a] ? J.n[a] : J.n[a] - 2; }
 
-// Work-list tables of the fused stage for tile height ty and k-chunk kc
+// Form of the fused stage a jet takes (0 general metrics, 1 product grid): a
+// separable handle's jets and those whose metrics are diagonal with positive
+// spacings (JetHost::diag).  Measured on the 384x256x144 jet, ms per stage:
+// general 0.951, product 0.543.
+static int form_of(const les_handle *h, int jet) { return h->sep || h->J[jet].diag ? 1 : 0; }
+
+// Work lists of form fi of the fused stage for tile height ty and k-chunk kc
 // (kc = 0: balanced form, items are tile-planes split evenly over the grid;
 // kc = -1: the same after waves of whole columns, in lockstep).
-static int set_fused_tiling(les_handle *h, int ty, int kc)
+static int set_fused_tiling(les_handle *h, int fi, int ty, int kc)
 {
+    les_handle::Form &M = h->form[fi];
     int acc = 0, tiles = 0;
     std::vector<FusedJet> one(h->njets);
     for (int j = 0; j < h->njets; ++j) {
-        FusedJet &F = h->fj[j];
+        FusedJet &F = M.fj[j];
         const JetHost &J = h->J[j];
         F.nbx = (out_len(J, 0) + 29) / 30;
-        F.nby = (out_len(J, 1) + ty - 3) / (ty - 2);
+        F.nby = form_of(h, j) == fi ? (out_len(J, 1) + ty - 3) / (ty - 2) : 0;
         if (kc <= 0) {
             F.kc = 0;
             F.nkc = out_len(J, 2); // planes per column: the items are tile-planes
@@ -494,14 +510,14 @@ static int set_fused_tiling(les_handle *h, int ty, int kc)
         one[j].item0 = 0;
         one[j].tile0 = 0;
     }
-    h->fused_ty = ty;
-    h->fused_balanced = kc == 0 ? 1 : (kc < 0 ? 2 : 0);
-    h->fused_items = acc;
-    h->fused_tiles = tiles;
-    CK(cudaMemcpyAsync(h->d_fj, h->fj.data(), sizeof(FusedJet) * h->njets, cudaMemcpyHostToDevice, h->st));
-    CK(cudaMemcpyAsync(h->d_fj1, one.data(), sizeof(FusedJet) * h->njets, cudaMemcpyHostToDevice, h->st));
+    M.ty = ty;
+    M.balanced = kc == 0 ? 1 : (kc < 0 ? 2 : 0);
+    M.items = acc;
+    M.tiles = tiles;
+    CK(cudaMemcpyAsync(M.d_fj, M.fj.data(), sizeof(FusedJet) * h->njets, cudaMemcpyHostToDevice, h->st));
+    CK(cudaMemcpyAsync(M.d_fj1, one.data(), sizeof(FusedJet) * h->njets, cudaMemcpyHostToDevice, h->st));
     CK(cudaStreamSynchronize(h->st));
-    h->fj1 = one;
+    M.fj1 = one;
     return LES_OK;
 }
 
@@ -512,26 +528,40 @@ static std::string kc_label(int kc)
 }
 static int autotune_fused(les_handle *h);
 
-// One fused stage (or residual) over all jets (jet < 0) or one jet.
-static void fused_launch(les_handle *h, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st)
+// One form's launch of a fused stage (or residual) over all its jets (jet < 0)
+// or one jet.
+static void fused_launch_form(les_handle *h, int fi, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st)
 {
+    const les_handle::Form &M = h->form[fi];
     const JetDev<float> *jets = (const JetDev<float> *)h->d_jets;
-    const FusedJet *fj = jet < 0 ? h->d_fj : h->d_fj1 + jet;
+    const FusedJet *fj = jet < 0 ? M.d_fj : M.d_fj1 + jet;
     const int nj = jet < 0 ? h->njets : 1;
-    const int items = jet < 0 ? h->fused_items : items_of(h->fj[jet]);
-    const int tiles = jet < 0 ? h->fused_tiles : h->fj[jet].nbx * h->fj[jet].nby;
-    const int grid = std::max(1, std::min(items, h->nsm * h->fused_cps[h->fused_ty == 16 ? 1 : 0]));
-    if (jet >= 0) jets += jet;
-    const int bal = h->fused_balanced;
+    const int items = jet < 0 ? M.items : items_of(M.fj[jet]);
+    const int tiles = jet < 0 ? M.tiles : M.fj[jet].nbx * M.fj[jet].nby;
+    const int grid = std::max(1, std::min(items, h->nsm * M.cps[M.ty / 8 - 1]));
+    const double *dt = h->d_dt;
+    if (jet >= 0) {
+        jets += jet;
+        dt += jet;
+    }
     // a single jet's table entries travel as kernel parameters
     const JetDev<float> *j1 = nj == 1 ? &h->jd32[jet < 0 ? 0 : jet] : nullptr;
-    const FusedJet *f1 = nj == 1 ? (jet < 0 ? &h->fj[0] : &h->fj1[jet]) : nullptr;
-    if (h->fused_ty == 16)
-        launch_fused<16>(jets, fj, nj, items, tiles, grid, src, dst, stage, h->d_dt, rhs_only, h->sep, bal,
-                         h->stage_wait_limit, j1, f1, st);
-    else
-        launch_fused<8>(jets, fj, nj, items, tiles, grid, src, dst, stage, h->d_dt, rhs_only, h->sep, bal,
-                         h->stage_wait_limit, j1, f1, st);
+    const FusedJet *f1 = nj == 1 ? (jet < 0 ? &M.fj[0] : &M.fj1[jet]) : nullptr;
+    const FusedLaunch a{jets, fj, nj, items, tiles, src, dst, stage, dt, rhs_only, M.balanced, h->stage_wait_limit};
+    if (fi == 1) launch_fused_prod(M.ty, a, grid, j1, f1, st);
+    else launch_fused(M.ty, a, grid, j1, f1, st);
+}
+
+// The same for every form in use; returns the number of launches.
+static int fused_launch(les_handle *h, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st)
+{
+    int n = 0;
+    for (int fi = 0; fi < 2; ++fi)
+        if (jet < 0 ? h->form[fi].any : form_of(h, jet) == fi) {
+            fused_launch_form(h, fi, jet, src, dst, stage, rhs_only, st);
+            ++n;
+        }
+    return n;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (the
@@ -555,18 +585,18 @@ static EncodeTiledFn encode_tiled()
 }
 
 // TMA maps of one FP32 jet's three state registers for the fused stage's
-// staging box (5 fields x 1 plane x (TY + 4) rows x 40 columns) at TY = 8 and
-// 16: tensor [field][k][j][i] with the padded row and field strides, columns
+// staging box (5 fields x 1 plane x (TY + 4) rows x 40 columns) at TY = 8, 16
+// and 24: tensor [field][k][j][i] with the padded row and field strides, columns
 // beyond ni read as zero.  Returns false if the encoder refuses.
-static bool make_state_maps(const JetHost &J, CUtensorMap out[6])
+static bool make_state_maps(const JetHost &J, CUtensorMap out[9])
 {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const cuuint64_t dims[4] = {(cuuint64_t)J.n[0], (cuuint64_t)J.n[1], (cuuint64_t)J.n[2], 5};
     const cuuint64_t strides[3] = {(cuuint64_t)J.pitch * 4, (cuuint64_t)J.pitch * J.n[1] * 4, (cuuint64_t)J.fs * 4};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    for (int t = 0; t < 2; ++t) {
-        const cuuint32_t box[4] = {(cuuint32_t)TMA_BOX_X, (cuuint32_t)tma_box_rows(t == 0 ? 8 : 16), 1, 5};
+    for (int t = 0; t < 3; ++t) {
+        const cuuint32_t box[4] = {(cuuint32_t)TMA_BOX_X, (cuuint32_t)tma_box_rows(8 * (t + 1)), 1, 5};
         for (int r = 0; r < 3; ++r)
             if (enc(&out[3 * t + r], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, J.q[r], dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -644,10 +674,12 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
     h->d_diag = (double *)(B + GP.o_diag);
     h->d_probe_base = (long long *)(B + GP.o_pbase);
     h->d_stage = (double *)(B + GP.o_stage);
-    h->d_fj = (FusedJet *)(B + GP.o_fj);
+    for (int f = 0; f < 2; ++f) {
+        h->form[f].d_fj = (FusedJet *)(B + GP.o_fj) + 2 * (size_t)f * njets;
+        h->form[f].d_fj1 = h->form[f].d_fj + njets;
+    }
     h->d_oob = (unsigned long long *)(B + GP.o_oob);
     h->d_tmap = (CUtensorMap *)(B + GP.o_tmap);
-    h->d_fj1 = h->d_fj + njets;
     for (int j = 0; j < njets; ++j) {
         JetHost &J = h->J[j];
         char *jb = B + gbytes + J.off;
@@ -675,13 +707,16 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
     CK(cudaMemcpyAsync(h->d_jets, D.data(), sizeof(JetDev<real>) * njets, cudaMemcpyHostToDevice, h->st));
     if constexpr (sizeof(real) == sizeof(float)) h->jd32 = D;
     if (h->prec == LES_FP32) {
-        if (fused_prepare<16>() != 0 || fused_prepare<8>() != 0)
+        if (fused_prepare<16>() != 0 || fused_prepare<8>() != 0 || fused_prod_prepare() != 0)
             return bail(fail(h, LES_ERR_CUDA, "fused kernel shared-memory attribute"));
-        h->fused_cps[0] = fused_ctas_per_sm(8, h->sep ? 1 : 0);
-        h->fused_cps[1] = fused_ctas_per_sm(16, h->sep ? 1 : 0);
-        h->fj.resize(njets);
+        for (int j = 0; j < njets; ++j) h->form[form_of(h, j)].any = true;
+        for (int t = 0; t < 3; ++t) {
+            if (t < 2) h->form[0].cps[t] = fused_ctas_per_sm(8 * (t + 1));
+            h->form[1].cps[t] = fused_prod_ctas_per_sm(8 * (t + 1));
+        }
+        std::vector<FusedJet> fj(njets);
         for (int j = 0; j < njets; ++j) {
-            FusedParams &F = h->fj[j].fp;
+            FusedParams &F = fj[j].fp;
             const les_params &pp = h->J[j].prm;
             F.gam = (float)pp.gamma;
             F.gm1 = (float)(pp.gamma - 1.0);
@@ -696,24 +731,27 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
             F.suthS = (float)S;
             F.cs2 = (float)(pp.Cs * pp.Cs);
             F.pinf = (float)(1.0 / pp.gamma);
-            for (int a = 0; a < 3; ++a) h->fj[j].h1[a] = h->J[j].h1[a];
-            h->fj[j].mp = h->J[j].mp;
-            h->fj[j].njp = (h->J[j].n[1] + 1) / 2;
-            h->fj[j].tmap = nullptr;
+            for (int a = 0; a < 3; ++a) fj[j].h1[a] = h->J[j].h1[a];
+            fj[j].mp = h->J[j].mp;
+            fj[j].njp = (h->J[j].n[1] + 1) / 2;
+            fj[j].tmap = nullptr;
         }
         // TMA maps for jets whose i and j axes are not periodic (a periodic
         // tile halo wraps, which a box cannot)
         {
-            std::vector<CUtensorMap> maps(6 * (size_t)njets);
+            std::vector<CUtensorMap> maps(9 * (size_t)njets);
             std::memset(maps.data(), 0, maps.size() * sizeof(CUtensorMap));
             for (int j = 0; j < njets; ++j)
-                if (!h->J[j].per[0] && !h->J[j].per[1] && make_state_maps(h->J[j], &maps[6 * (size_t)j]))
-                    h->fj[j].tmap = h->d_tmap + 6 * (size_t)j;
+                if (!h->J[j].per[0] && !h->J[j].per[1] && make_state_maps(h->J[j], &maps[9 * (size_t)j]))
+                    fj[j].tmap = h->d_tmap + 9 * (size_t)j;
             CK(cudaMemcpyAsync(h->d_tmap, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
                                h->st));
         }
-        int rc = set_fused_tiling(h, 8, 32);
-        if (rc) return bail(rc);
+        for (int f = 0; f < 2; ++f) {
+            h->form[f].fj = fj;
+            int rc = set_fused_tiling(h, f, 8, 32);
+            if (rc) return bail(rc);
+        }
     }
     // block maps: [pt | bc | ptg | ptp] each njets+1, then per-jet pairs
     std::vector<int> maps(MAP_FAMS * (njets + 1) + 2 * MAP_FAMS * njets);
@@ -873,9 +911,8 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
         if (h->prec == LES_FP32) {
             // fused single-pass stage: counted as the interface kernel kind
             T.begin(LES_KERNEL_IFACE);
-            fused_launch(h, -1, src_of[s], dst_of[s], s, 0, st);
+            h->launches_per_step += fused_launch(h, -1, src_of[s], dst_of[s], s, 0, st);
             T.end();
-            h->launches_per_step += 1;
             if (h->bcm.total > 0) { // none on a fully periodic grid
                 T.begin(LES_KERNEL_BC);
                 h->launches_per_step += bc_pass<real>(h, h->bcm, jets, dst_of[s], st);
@@ -1112,12 +1149,15 @@ struct EventPair { // destroyed on every return path
 };
 } // namespace
 
-static int autotune_fused(les_handle *h)
+static int autotune_form(les_handle *h, int fi)
 {
-    std::string key = "dev" + std::to_string(h->dev) + ":";
-    for (auto &J : h->J)
+    std::string key = "dev" + std::to_string(h->dev) + (fi ? "p:" : "g:");
+    for (int j = 0; j < h->njets; ++j) {
+        if (form_of(h, j) != fi) continue;
+        const JetHost &J = h->J[j];
         key += std::to_string(J.n[0]) + "x" + std::to_string(J.n[1]) + "x" + std::to_string(J.n[2]) + "p" +
-               std::to_string(J.per[0] * 4 + J.per[1] * 2 + J.per[2]) + (h->sep ? "s;" : ";");
+               std::to_string(J.per[0] * 4 + J.per[1] * 2 + J.per[2]) + ";";
+    }
     std::pair<int, int> pick{8, 48};
     bool cached = false;
     {
@@ -1129,37 +1169,45 @@ static int autotune_fused(les_handle *h)
         }
     }
     if (!cached) {
-        const int tys[2] = {16, 8};
+        const int tys[3] = {16, 8, 24}; // 24: product form only
         // 0: balanced tile-plane ranges; -1: whole-column waves, then balanced ranges
         const int kcs[8] = {8, 16, 24, 48, 96, 100000, 0, -1};
         float best = 1e30f;
         EventPair ev;
         CK(cudaEventCreate(&ev.e0));
         CK(cudaEventCreate(&ev.e1));
-        for (int ty : tys)
+        for (int t = 0; t < (fi ? 3 : 2); ++t)
             for (int kc : kcs) {
-                int rc = set_fused_tiling(h, ty, kc);
+                int rc = set_fused_tiling(h, fi, tys[t], kc);
                 if (rc) return rc;
                 // real stage launches from Q(0) into the first stage register,
                 // which holds no state between steps
-                fused_launch(h, -1, 0, 1, 0, 0, h->st); // warm-up
+                fused_launch_form(h, fi, -1, 0, 1, 0, 0, h->st); // warm-up
                 CK(cudaEventRecord(ev.e0, h->st));
-                for (int rep = 0; rep < 3; ++rep) fused_launch(h, -1, 0, 1, 0, 0, h->st);
+                for (int rep = 0; rep < 3; ++rep) fused_launch_form(h, fi, -1, 0, 1, 0, 0, h->st);
                 CK(cudaEventRecord(ev.e1, h->st));
                 CK(cudaEventSynchronize(ev.e1));
                 float ms = 0;
                 CK(cudaEventElapsedTime(&ms, ev.e0, ev.e1));
                 if (ms < best) {
                     best = ms;
-                    pick = {ty, kc};
+                    pick = {tys[t], kc};
                 }
             }
         std::lock_guard<std::mutex> lk(g_tune_mu);
         pick = g_tune_cache.emplace(key, pick).first->second;
     }
-    h->tune_note = "ty=" + std::to_string(pick.first) + " kc=" + kc_label(pick.second) +
-                   " (tuned over ty {16,8} x kc {8,16,24,48,96,all,balanced,lockstep})";
-    return set_fused_tiling(h, pick.first, pick.second);
+    h->form[fi].note = "ty=" + std::to_string(pick.first) + " kc=" + kc_label(pick.second) + " (tuned over ty " +
+                       (fi ? "{16,8,24}" : "{16,8}") + " x kc {8,16,24,48,96,all,balanced,lockstep})";
+    return set_fused_tiling(h, fi, pick.first, pick.second);
+}
+
+static int autotune_fused(les_handle *h)
+{
+    for (int fi = 0; fi < 2; ++fi)
+        if (h->form[fi].any)
+            if (int rc = autotune_form(h, fi)) return rc;
+    return LES_OK;
 }
 
 template <typename real> static int diag_impl(les_handle *h, int jet, les_diag *d)
@@ -1270,11 +1318,12 @@ extern "C" int les_set_fused_tiling(les_handle *h, int ty, int kc)
     if (!h) return LES_ERR_ARG;
     if (h->prec != LES_FP32) return fail(h, LES_ERR_ARG, "the fused tiling applies to FP32 handles");
     if ((ty != 8 && ty != 16) || kc < -1) return fail(h, LES_ERR_ARG, "ty must be 8 or 16 and kc >= -1");
-    int rc = set_fused_tiling(h, ty, kc);
-    if (rc) return rc;
+    for (int fi = 0; fi < 2; ++fi) {
+        int rc = set_fused_tiling(h, fi, ty, kc);
+        if (rc) return rc;
+        h->form[fi].note = "ty=" + std::to_string(ty) + " kc=" + kc_label(kc) + " (set by the caller)";
+    }
     h->tuned = true;
-    h->tune_note = "ty=" + std::to_string(ty) + " kc=" + kc_label(kc) +
-                   " (set by the caller)";
     if (h->gexec) { // the captured step holds the old work list
         cudaGraphExecDestroy(h->gexec);
         h->gexec = nullptr;
@@ -1372,10 +1421,22 @@ extern "C" const char *les_describe(les_handle *h)
     if (!h) return "null handle";
     static thread_local std::string d;
     d = std::string(h->prec == LES_FP64 ? "fp64" : "fp32") + " jets=" + std::to_string(h->njets) +
-        " device_bytes=" + std::to_string(h->bytes) + " stage=" +
-        (h->prec == LES_FP64 ? std::string("point+grads+iface+update") + (h->ptg.total == 0 ? " (product)" : h->ptp.total > 0 ? " (general, product)" : " (general)")
-                             : std::string(h->sep ? "fused separable " : "fused ") + (h->tuned ? h->tune_note : "ty=" + std::to_string(h->fused_ty) + " (untuned)")) +
-        " launches_per_step=" + std::to_string(h->launches_per_step);
+        " device_bytes=" + std::to_string(h->bytes) + " stage=";
+    if (h->prec == LES_FP64) {
+        d += "point+grads+iface+update";
+        d += h->ptg.total == 0 ? " (product)" : (h->ptp.total > 0 ? " (general, product)" : " (general)");
+    } else {
+        bool first = true;
+        for (int fi = 1; fi >= 0; --fi) {
+            const les_handle::Form &M = h->form[fi];
+            if (!M.any) continue;
+            d += first ? "fused " : " + fused ";
+            d += fi == 0 ? "general " : (h->sep ? "product (separable) " : "product ");
+            d += h->tuned ? M.note : "ty=" + std::to_string(M.ty) + " (untuned)";
+            first = false;
+        }
+    }
+    d += " launches_per_step=" + std::to_string(h->launches_per_step);
     return d.c_str();
 }
 

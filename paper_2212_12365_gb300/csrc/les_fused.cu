@@ -1,4 +1,5 @@
-// Fused single-pass Runge-Kutta stage for FP32 storage and arithmetic.
+// Fused single-pass Runge-Kutta stage for FP32 storage and arithmetic, general
+// metrics (jets on a product grid take les_fused_prod.cu).
 //
 // One kernel does what k_point, k_grads, k_iface and k_update do for the FP64
 // path (Secs. "Numerical Formulation", "Time Marching Method"), with the
@@ -18,7 +19,7 @@
 // (rows 2tr|2tr+1 and 2tr+1|2tr+2) take their right-hand points from its own
 // second row and the next thread row's first.
 //
-// Halo.  Point data (primitives and rho H) live in a ring of 4 planes over
+// Halo.  Point data (primitives and rho H) live in a ring of 3 planes over
 // R2 = R1 plus one column on each side and two rows above and below; cells
 // outside a non-periodic axis hold the mirror image of the point one beyond
 // the boundary point (W(-1) = W(1), W(n) = W(n-2)), which is the paper's
@@ -36,67 +37,31 @@
 #include <algorithm>
 #include <cmath>
 
-#include "les_internal.cuh"
+#include "les_fused.cuh"
 
 namespace les {
 
 namespace {
 
-constexpr int FX = 32; // threads (grid columns) along i
-
-__constant__ float c_alpha_f[5] = {0.25f, 1.0f / 6.0f, 0.375f, 0.5f, 1.0f};
-
-// ---------------------------------------------------------------------------
-// Paired FP32 arithmetic (two rows per register pair)
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 bc(float s) { return make_float2(s, s); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// a - b, rounded once like a scalar subtraction
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, bc(-1.0f), a); }
-__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
-__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
-__device__ __forceinline__ float4 cat4(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
-// the pair (second lane of a, first lane of b): the +eta neighbours of a
-// thread's two rows
-__device__ __forceinline__ float2 odd2(float2 a, float2 b) { return make_float2(a.y, b.x); }
-__device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-// hardware approximate reciprocal (positive, normal arguments)
-__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)); }
-// square root of x >= 0 through the hardware reciprocal square root
-// (max. 2 ulp): x * rsqrt(x), 0 -> 0 (a spectral radius vanishes on the axis
-// of a polar mesh)
-__device__ __forceinline__ float2 sqrt2(float2 x)
-{
-    return mul2(x, make_float2(rsqrtf(fmaxf(x.x, 1.17549435e-38f)), rsqrtf(fmaxf(x.y, 1.17549435e-38f))));
-}
-
 // ---------------------------------------------------------------------------
 // Shared-memory map (byte offsets; 16-byte records first)
-//   ring (3 planes; 4 separable) over R2 pair cells:  PA (rho, u)  PB (v, w)  PC (p, T)
+//   ring (3 planes) over R2 pair cells:  PA (rho, u)  PB (v, w)  PC (p, T)
 //                                         float4 each; PH (rho H) float2
 //   R1 tables (2 planes) over R1 pair cells:
 //     GD [3 axes][2]  float4: 2 d/d xi^a of (u, v) and (w, T)
 //     GC [4]          float4: (mu_eff, kappa), (nu_a, lambda-bar_a) a = 0..2
 //   MA [3 planes][5] float4 over R1 pair cells: cofactors (m0 m1) (m2 m3)
 //                             (m4 m5) (m6 m7) (m8 J^-1), streamed in by
-//                             cp.async one plane ahead (general form only)
+//                             cp.async one plane ahead
 //   SH [5][NT] float          eta flux of each thread's second row
 //   QZ [5][TY-2][30] float    Q(0) of the tile's updated points, copied in
 //                             by cp.async during the plane's iteration
-//   HX [C2], HY [TY+4] float4 separable form: (h, 1/h, h^(2/3), 0) of the
-//                             tile's columns / rows
-//   HZ [4] float4             separable form: the same for planes k (slot k & 3),
-//                             copied in two planes ahead
 //   QG [5][TY+4][40] float    the next plane's state box (TMA), 128-aligned,
 //                             then its mbarrier
 // A "pair cell" is one column of two rows (2p, 2p+1); its float4 records
 // interleave the two rows: (q1(2p), q1(2p+1), q2(2p), q2(2p+1)).
 // ---------------------------------------------------------------------------
-template <int TY, bool SEP> struct Geo {
+template <int TY> struct Geo {
     static constexpr int TR = TY / 2;              // thread rows
     static constexpr int NT = FX * TR;             // threads
     static constexpr int C2 = FX + 2;              // R2 columns -1 .. FX
@@ -104,9 +69,7 @@ template <int TY, bool SEP> struct Geo {
     static constexpr int N2 = C2 * P2;             // R2 pair cells
     static constexpr int N1 = NT;                  // R1 pair cells
     static constexpr int BR = tma_box_rows(TY);    // rows of the staging box
-    // planes of the point ring: 3 in the general form (its shared memory
-    // also holds three planes of metric records), 4 in the separable form
-    static constexpr int NR = SEP ? 4 : 3;
+    static constexpr int NR = 3;                   // planes of the point ring
     static constexpr size_t O_PA = 0;
     static constexpr size_t O_PB = O_PA + 16ull * NR * N2;
     static constexpr size_t O_PC = O_PB + 16ull * NR * N2;
@@ -114,14 +77,10 @@ template <int TY, bool SEP> struct Geo {
     static constexpr size_t O_GD = O_PH + 8ull * NR * N2;
     static constexpr size_t O_GC = O_GD + 16ull * 2 * 6 * N1;
     static constexpr size_t O_MA = O_GC + 16ull * 2 * 4 * N1;
-    static constexpr size_t O_SH = O_MA + (SEP ? 0ull : 16ull * 3 * 5 * N1);
+    static constexpr size_t O_SH = O_MA + 16ull * 3 * 5 * N1;
     static constexpr int QZN = (TY - 2) * (FX - 2); // updated points of a tile plane
     static constexpr size_t O_QZ = (O_SH + 4ull * 5 * NT + 15) / 16 * 16;
-    static constexpr size_t O_HX = O_QZ + 4ull * 5 * QZN;
-    // (the spacing tables exist in the separable form only)
-    static constexpr size_t O_HY = O_HX + (SEP ? 16ull * C2 : 0ull);
-    static constexpr size_t O_HZ = O_HY + (SEP ? 16ull * BR : 0ull);
-    static constexpr size_t O_QG = (O_HZ + (SEP ? 16ull * 4 : 0ull) + 127) / 128 * 128;
+    static constexpr size_t O_QG = (O_QZ + 4ull * 5 * QZN + 127) / 128 * 128;
     static constexpr unsigned BOX_BYTES = 4u * 5 * BR * TMA_BOX_X;
     static_assert(BOX_BYTES % 16 == 0, "box size");
     static constexpr size_t O_MBAR = O_QG + BOX_BYTES;
@@ -130,101 +89,28 @@ template <int TY, bool SEP> struct Geo {
     static_assert(BYTES <= 227 * 1024, "shared memory of one CTA");
 };
 
-template <int TY, bool SEP> struct Sm {
+template <int TY> struct Sm {
     float4 *PA, *PB, *PC;
     float2 *PH;
     float4 *GD, *GC, *MA;
     float *SH, *QZ;
-    float4 *HX, *HY, *HZ;
     float *QG;
     unsigned long long *MBAR;
     float *FPS; // a batch jet's constants (FusedParams) for the item
     __device__ __forceinline__ explicit Sm(unsigned char *b)
-        : PA((float4 *)(b + Geo<TY, SEP>::O_PA)), PB((float4 *)(b + Geo<TY, SEP>::O_PB)),
-          PC((float4 *)(b + Geo<TY, SEP>::O_PC)), PH((float2 *)(b + Geo<TY, SEP>::O_PH)),
-          GD((float4 *)(b + Geo<TY, SEP>::O_GD)), GC((float4 *)(b + Geo<TY, SEP>::O_GC)),
-          MA((float4 *)(b + Geo<TY, SEP>::O_MA)), SH((float *)(b + Geo<TY, SEP>::O_SH)),
-          QZ((float *)(b + Geo<TY, SEP>::O_QZ)),
-          HX((float4 *)(b + Geo<TY, SEP>::O_HX)), HY((float4 *)(b + Geo<TY, SEP>::O_HY)),
-          HZ((float4 *)(b + Geo<TY, SEP>::O_HZ)),
-          QG((float *)(b + Geo<TY, SEP>::O_QG)), MBAR((unsigned long long *)(b + Geo<TY, SEP>::O_MBAR)),
-          FPS((float *)(b + Geo<TY, SEP>::O_FPS))
+        : PA((float4 *)(b + Geo<TY>::O_PA)), PB((float4 *)(b + Geo<TY>::O_PB)),
+          PC((float4 *)(b + Geo<TY>::O_PC)), PH((float2 *)(b + Geo<TY>::O_PH)),
+          GD((float4 *)(b + Geo<TY>::O_GD)), GC((float4 *)(b + Geo<TY>::O_GC)),
+          MA((float4 *)(b + Geo<TY>::O_MA)), SH((float *)(b + Geo<TY>::O_SH)),
+          QZ((float *)(b + Geo<TY>::O_QZ)),
+          QG((float *)(b + Geo<TY>::O_QG)), MBAR((unsigned long long *)(b + Geo<TY>::O_MBAR)),
+          FPS((float *)(b + Geo<TY>::O_FPS))
     {
     }
 };
 
 // Slot of plane k (k >= -6) in the three-plane rings.
 __device__ __forceinline__ int r3(int k) { return (k + 6) % 3; }
-// Slot of plane k in the point ring of NR planes.
-template <int NR> __device__ __forceinline__ int rslot(int k) { return NR == 4 ? (k & 3) : r3(k); }
-
-// Asynchronous 16-byte global -> shared copy, not kept in L1 (completes
-// without the issuing thread waiting; cp_async_wait_prev() waits for all of
-// this thread's groups but the most recent one).
-__device__ __forceinline__ unsigned smem_u32_(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32_(dst)), "l"(src) : "memory");
-}
-// 4-byte variant (scattered Q(0) values)
-__device__ __forceinline__ void cp_async4(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_u32_(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// Index of a tile cell along an axis: wrapped on a periodic axis; on a
-// non-periodic one the mirror image about the end point (-g, 2(n-1) - g),
-// clamped into the axis for cells further out (those feed no result).
-__device__ __forceinline__ int map_idx(int g, int n, int per)
-{
-    if (per) {
-        const int h = g < 0 ? g + n : (g >= n ? g - n : g);
-        return (unsigned)h < (unsigned)n ? h : wrapi(g, n);
-    }
-    const int m = g < 0 ? -g : (g > n - 1 ? 2 * (n - 1) - g : g);
-    return m < 0 ? 0 : (m > n - 1 ? n - 1 : m);
-}
-
-// TMA staging: an mbarrier with one arrival (the issuing thread's, carrying
-// the expected byte count) completed by the copy.
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long *bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); // visible to the copy engine
-}
-// 4-D tiled copy (x, y, z, field) of the tensor map's box into shared memory;
-// x must be a multiple of 4 elements (16 bytes); other coordinates may lie
-// outside the tensor (zero fill).
-__device__ __forceinline__ void tma_box_load(float *dst, const CUtensorMap *map, int x, int y, int z,
-                                             unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                 " [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(smem_u32(dst)),
-                 "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(z), "r"(0), "r"(smem_u32(bar))
-                 : "memory");
-}
-// Wait for the phase of the given parity, polling at most `limit` times
-// (false: gave up).
-constexpr int MBAR_WAIT_LIMIT = 1 << 22;
-__device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity, int limit)
-{
-    for (int it = 0; it < limit; ++it) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(smem_u32(bar)), "r"(parity)
-                     : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 // Point data of one side of an interface: two points (the two lanes).
 struct Pts {
@@ -357,65 +243,6 @@ __device__ __forceinline__ void iface(const FusedParams &FP, const Pts &L, const
     }
 }
 
-// Separable form of iface on a Cartesian-product grid x = x(i), y = y(j),
-// z = z(k) (Sec. "Transformation of Coordinates" with diagonal metrics): the
-// cofactor matrix is diag(y_eta z_zeta, x_xi z_zeta, x_xi y_eta), so the face
-// factor Sa of axis A is the product of the two tangential spacings (equal on
-// both sides), the interface J^-1 is Sa hb with hb the average spacing along
-// A, and the chain rule is d/dx_c = (1/h_c) d/dxi_c.  rhb = 1/hb; rq1, rq2:
-// 1/4 of the reciprocal tangential spacings (axes B1 < B2), which turn the
-// sums of doubled differences into derivatives.
-template <int A>
-__device__ __forceinline__ void iface_sep(const FusedParams &FP, const Pts &L, const float2 WL[5], const Pts &R,
-                                          const float2 WR[5], const float2 WLm[5], const float2 WRp[5],
-                                          const Side &SL, const Side &SR, float2 Sa, float2 hb, float2 rhb,
-                                          float2 rq1, float2 rq2, float2 H[5])
-{
-    const float2 half = bc(0.5f);
-    const float2 hS = mul2(half, Sa);
-    // centred inviscid flux: J^-1 U_A = Sa u_A on both sides
-    const float2 uAL = A == 0 ? L.u : (A == 1 ? L.v : L.w), uAR = A == 0 ? R.u : (A == 1 ? R.v : R.w);
-    const float2 hJL = mul2(hS, uAL), hJR = mul2(hS, uAR);
-#pragma unroll
-    for (int f = 0; f < 5; ++f) H[f] = fma2(WR[f], hJR, mul2(WL[f], hJL));
-    H[1 + A] = fma2(hS, sub2(add2(L.p, R.p), bc(2.0f * FP.pinf)), H[1 + A]); // ambient pressure out, as above
-    // Turkel-Vatsa dissipation
-    {
-        const float2 eps2 = mul2(bc(FP.k2), max2(SL.nu, SR.nu));
-        const float2 eps4 = max2(bc(0.0f), sub2(bc(FP.k4), eps2));
-        const float2 sc = mul2(mul2(hS, hb), add2(SL.lb, SR.lb)); // Sa hb (lb_L + lb_R) / 2
-        const float2 se4 = mul2(sc, eps4);
-        const float2 c2 = fma2(se4, bc(3.0f), mul2(sc, eps2));
-#pragma unroll
-        for (int f = 0; f < 5; ++f) H[f] = fma2(c2, sub2(WL[f], WR[f]), fma2(se4, sub2(WRp[f], WLm[f]), H[f]));
-    }
-    // compact viscous + SGS flux: only row A of the stress tensor is needed
-    {
-        float2 g[4][3]; // physical gradient of (u, v, w, T) at the interface
-        constexpr int B1 = A == 0 ? 1 : 0, B2 = A == 2 ? 1 : 2;
-        g[0][A] = mul2(sub2(R.u, L.u), rhb);
-        g[1][A] = mul2(sub2(R.v, L.v), rhb);
-        g[2][A] = mul2(sub2(R.w, L.w), rhb);
-        g[3][A] = mul2(sub2(R.T, L.T), rhb);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            g[f][B1] = mul2(add2(SL.d[0][f], SR.d[0][f]), rq1);
-            g[f][B2] = mul2(add2(SL.d[1][f], SR.d[1][f]), rq2);
-        }
-        const float2 coef = mul2(half, add2(SL.mue, SR.mue)); // mu_eff at the interface
-        const float2 dv3 = mul2(bc(2.0f / 3.0f), add2(add2(g[0][0], g[1][1]), g[2][2]));
-        float2 tA[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-            tA[i] = i == A ? mul2(coef, sub2(add2(g[A][A], g[A][A]), dv3)) : mul2(coef, add2(g[A][i], g[i][A]));
-        const float2 kap = mul2(half, add2(SL.kap, SR.kap));
-#pragma unroll
-        for (int i = 0; i < 3; ++i) H[1 + i] = sub2(H[1 + i], mul2(Sa, tA[i]));
-        const float2 e = fma2(tA[2], add2(L.w, R.w), fma2(tA[1], add2(L.v, R.v), mul2(tA[0], add2(L.u, R.u))));
-        H[4] = sub2(H[4], mul2(Sa, fma2(kap, g[3][A], mul2(half, e))));
-    }
-}
-
 } // namespace
 
 // Index checks of a LES_BOUNDS_CHECK build (nothing otherwise): global
@@ -423,42 +250,21 @@ __device__ __forceinline__ void iface_sep(const FusedParams &FP, const Pts &L, c
 // shared-memory slots against their tables (5 point ring, 6 R1 tables and
 // the staging box, 7 eta-flux rows).
 #define CK_G(site, x, n) LES_BOUNDS(J.oob, (site), (x), (n))
-#define CK_RING(x) ((int)LES_BOUNDS(J.oob, 5, (x), NRING * N2))
+#define CK_RING(x) ((int)LES_BOUNDS(J.oob, 5, (x), G_::NR * N2))
 #define CK_TAB(x, n) ((int)LES_BOUNDS(J.oob, 6, (x), (n)))
 #define CK_SH(x) ((int)LES_BOUNDS(J.oob, 7, (x), 5 * NT))
 
-// The jet's table entries: in the single-jet form (ONE) the kernel
-// parameters, whose fields the compiler reads from the parameter bank
-// (warp-uniform operands, no memory loads in the plane loop); else the
-// device tables.
-template <bool ONE, typename T> __device__ __forceinline__ const T &jet_entry(const T &one, const T *tab, int j)
-{
-    if constexpr (ONE) return one;
-    else return tab[j];
-}
-
-// The jet's constants: the kernel parameter (ONE), else the item's copy in
-// shared memory (read with broadcast loads instead of global loads).
-template <bool ONE>
-__device__ __forceinline__ const FusedParams &jet_params(const FusedParams &param, const float *staged)
-{
-    if constexpr (ONE) return param;
-    else return *reinterpret_cast<const FusedParams *>(staged);
-}
-static_assert(sizeof(FusedParams) % 4 == 0 && sizeof(FusedParams) <= 64, "FusedParams staging");
-
-template <int TY, bool SEP, bool ONE>
+template <int TY, bool ONE>
 __global__ void __launch_bounds__(FX * TY / 2, 1)
     k_fused(const JetDev<float> *__restrict__ jets, const FusedJet *__restrict__ fj, int njets,
             int total_items, int total_tiles, int src, int dst, int stage, const double *__restrict__ dt,
             int rhs_only, int balanced, int wait_limit, const __grid_constant__ JetDev<float> j1,
             const __grid_constant__ FusedJet f1)
 {
-    using G_ = Geo<TY, SEP>;
+    using G_ = Geo<TY>;
     constexpr int TR = G_::TR, NT = G_::NT, C2 = G_::C2, N2 = G_::N2, N1 = G_::N1, BR = G_::BR;
-    constexpr int NRING = G_::NR;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const Sm<TY, SEP> S(smem_raw);
+    const Sm<TY> S(smem_raw);
     const int tx = threadIdx.x, tr = threadIdx.y;
     const int tid = tr * FX + tx;
     const int c1 = tid;                       // own R1 pair cell
@@ -632,16 +438,6 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                 bo[t][h] = rr * TMA_BOX_X + cl;
             }
         }
-        if constexpr (SEP) {
-            // 1-D spacings of the tile's columns and rows (the previous item's
-            // last reads of HX/HY precede its closing barrier)
-            if (tid < C2) {
-                S.HX[tid] = F.h1[0][map_idx(ib - 1 + tid, ni, pi)];
-            } else if (tid < C2 + BR) {
-                const int t = tid - C2;
-                S.HY[t] = F.h1[1][map_idx(jb - 2 + t, nj, pj)];
-            }
-        }
         // carried from plane to plane: the zeta flux below, W of the own
         // column one plane below the interface plane, J of the next update
         float2 hz_prev[5], Wc[5];
@@ -651,7 +447,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             Wc[f] = bc(0.0f);
         }
         float2 rjU = bc(0.0f), rjG = bc(0.0f);
-        __syncthreads(); // shared memory of the previous item is free; HX/HY written
+        __syncthreads(); // shared memory of the previous item is free
 
         // thread 0 issues the box of plane kq once every thread is done with
         // the previous one (after a barrier)
@@ -700,10 +496,8 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
         //      three-plane ring slots q3, q3m, q3p of planes kg, kg - 1, kg + 1) ----
         auto grad = [&](int kg, int gk, int q3, int q3m, int q3p) {
             // ring slots of planes kg, kg - 1 (= kg + 2), kg + 1 (= kg - 2)
-            const int sl0 = NRING == 4 ? (kg & 3) : q3;
-            const int slm = NRING == 4 ? ((kg - 1) & 3) : q3m, slp = NRING == 4 ? ((kg + 1) & 3) : q3p;
-            const int slm2 = NRING == 4 ? ((kg - 2) & 3) : q3p, slp2 = NRING == 4 ? ((kg + 2) & 3) : q3m;
-            const int s0 = sl0 * N2;
+            const int slm = q3m, slp = q3p, slm2 = q3p, slp2 = q3m;
+            const int s0 = q3 * N2;
             const int slot = kg & 1;
             const int own = CK_RING(s0 + c2);
             const float4 a0 = S.PA[own], b0 = S.PB[own], q0 = S.PC[own];
@@ -717,30 +511,10 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                 const float2 r = rcp2(den);
                 return make_float2(fabsf(num.x) * r.x, fabsf(num.y) * r.y);
             };
-            // Separable form: derivatives and sensor along xi or zeta in one
-            // instruction sequence for every lane, from the cells o1, o2 and the
-            // own cell with selected weights: central (t = 0: o1, o2 = c -+ 1,
-            // weights 0, -1, 1; sensor over o1, c, o2) or one-sided (o1, o2 =
-            // c + t, c + 2t, weights -3t, 4t, -t; sensor over c, o1, o2).  The
-            // same values as the branches of the general form below, which keeps
-            // the branches (its register budget is tighter; both measured).
-            auto axis3 = [&](int o1, int o2, int t, float2 dd[4], float2 &nn) {
-                const float4 a1 = S.PA[o1], b1 = S.PB[o1], q1 = S.PC[o1];
-                const float4 a2 = S.PA[o2], b2 = S.PB[o2], q2 = S.PC[o2];
-                const float tf = (float)t;
-                const float2 w0 = bc(-3.0f * tf), w1 = bc(t == 0 ? -1.0f : 4.0f * tf), w2 = bc(t == 0 ? 1.0f : -tf);
-                dd[0] = fma2(w2, hi2(a2), fma2(w1, hi2(a1), mul2(w0, U0[0])));
-                dd[1] = fma2(w2, lo2(b2), fma2(w1, lo2(b1), mul2(w0, U0[1])));
-                dd[2] = fma2(w2, hi2(b2), fma2(w1, hi2(b1), mul2(w0, U0[2])));
-                dd[3] = fma2(w2, hi2(q2), fma2(w1, hi2(q1), mul2(w0, T0)));
-                nn = sensor(t == 0 ? lo2(q1) : p0, t == 0 ? p0 : lo2(q1), lo2(q2));
-            };
             // along xi: central, or one-sided over the cells c, c+t, c+2t at a
             // non-periodic end (the sensor of an end point is its interior
             // neighbour's: same three points)
-            if constexpr (SEP) {
-                axis3(CK_RING(s0 + c2 + (ti == 0 ? -1 : ti)), CK_RING(s0 + c2 + (ti == 0 ? 1 : 2 * ti)), ti, d[0], nu[0]);
-            } else if (ti == 0) {
+            if (ti == 0) {
                 const int om = CK_RING(s0 + c2 - 1), op = CK_RING(s0 + c2 + 1);
                 const float4 am = S.PA[om], bm = S.PB[om], qm = S.PC[om];
                 const float4 ap = S.PA[op], bp = S.PB[op], qp = S.PC[op];
@@ -809,10 +583,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             // at an end of a non-periodic k axis
             {
                 const int tk = (!pk && gk == 0) ? 1 : ((!pk && gk == nk - 1) ? -1 : 0);
-                if constexpr (SEP) {
-                    axis3(CK_RING((tk == 0 ? slm : (tk > 0 ? slp : slm)) * N2 + c2),
-                          CK_RING((tk == 0 ? slp : (tk > 0 ? slp2 : slm2)) * N2 + c2), tk, d[2], nu[2]);
-                } else if (tk == 0) {
+                if (tk == 0) {
                     const int om = CK_RING(slm * N2 + c2), op = CK_RING(slp * N2 + c2);
                     const float4 am = S.PA[om], bm = S.PB[om], qm = S.PC[om];
                     const float4 ap = S.PA[op], bp = S.PB[op], qp = S.PC[op];
@@ -835,22 +606,8 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             }
             // metrics: cofactors m (rows of d xi^a / d x times J^-1), J,
             // (Cs Delta)^2 J, row norms
-            float2 m[9], rj, csdJ, nrm[3], rh[3];
-            if constexpr (SEP) {
-                // diagonal cofactors: 1/h_a per axis; J = prod 1/h_a
-                const float4 hX = S.HX[tx + 1];
-                const float4 hYA = S.HY[rA + 2], hYB = S.HY[rB + 2];
-                const float4 hZ = S.HZ[kg & 3];
-                rh[0] = bc(hX.y);
-                rh[1] = f2(hYA.y, hYB.y);
-                rh[2] = bc(hZ.y);
-                csdJ = mul2(bc(FP.cs2 * hX.z * hZ.z), f2(hYA.z, hYB.z)); // (Cs Delta)^2, Delta^3 = h_x h_y h_z
-                rj = mul2(bc(hX.y * hZ.y), rh[1]);
-#pragma unroll
-                for (int t = 0; t < 9; ++t) m[t] = bc(0.0f);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) nrm[a] = bc(0.0f);
-            } else {
+            float2 m[9], rj, csdJ, nrm[3];
+            {
                 float4 u[5];
 #pragma unroll
                 for (int q = 0; q < 5; ++q) u[q] = S.MA[CK_TAB((q3 * 5 + q) * N1 + c1, 15 * N1)];
@@ -866,19 +623,16 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     nrm[a] = sqrt2(fma2(m[3 * a + 2], m[3 * a + 2], fma2(m[3 * a + 1], m[3 * a + 1], mul2(m[3 * a], m[3 * a]))));
-                    rh[a] = bc(0.0f);
                 }
             }
-            // doubled physical velocity gradient g' (2 J^-1 du_i/dx_c for the
-            // general form, 2 du_i/dx_c separable), strain norm, Smagorinsky
+            // doubled physical velocity gradient g' = 2 J^-1 du_i/dx_c, strain norm,
+            // Smagorinsky
             float2 g[3][3];
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
-                for (int cc = 0; cc < 3; ++cc) {
-                    if constexpr (SEP) g[i][cc] = mul2(d[cc][i], rh[cc]);
-                    else g[i][cc] = fma2(m[6 + cc], d[2][i], fma2(m[3 + cc], d[1][i], mul2(m[cc], d[0][i])));
-                }
+                for (int cc = 0; cc < 3; ++cc)
+                    g[i][cc] = fma2(m[6 + cc], d[2][i], fma2(m[3 + cc], d[1][i], mul2(m[cc], d[0][i])));
             const float2 a01 = add2(g[0][1], g[1][0]), a02 = add2(g[0][2], g[2][0]), a12 = add2(g[1][2], g[2][1]);
             const float2 sd = fma2(g[2][2], g[2][2], fma2(g[1][1], g[1][1], mul2(g[0][0], g[0][0])));
             const float2 so = fma2(a12, a12, fma2(a02, a02, mul2(a01, a01)));
@@ -894,15 +648,9 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             float2 sq[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                float2 lam;
-                if constexpr (SEP) {
-                    const float2 ua = U0[a];
-                    lam = mul2(make_float2(fabsf(ua.x) + sT.x, fabsf(ua.y) + sT.y), rh[a]);
-                } else {
-                    const float2 JU = fma2(m[3 * a + 2], U0[2], fma2(m[3 * a + 1], U0[1], mul2(m[3 * a], U0[0])));
-                    lam = mul2(make_float2(fmaf(sT.x, nrm[a].x, fabsf(JU.x)), fmaf(sT.y, nrm[a].y, fabsf(JU.y))),
-                               rj);
-                }
+                const float2 JU = fma2(m[3 * a + 2], U0[2], fma2(m[3 * a + 1], U0[1], mul2(m[3 * a], U0[0])));
+                const float2 lam =
+                    mul2(make_float2(fmaf(sT.x, nrm[a].x, fabsf(JU.x)), fmaf(sT.y, nrm[a].y, fabsf(JU.y))), rj);
                 sq[a] = sqrt2(lam);
             }
             const float2 ssum = add2(add2(sq[0], sq[1]), sq[2]);
@@ -964,7 +712,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             // grid planes
             const int q3L = q3c, q3G = q3L == 0 ? 2 : q3L - 1, q3U = q3L == 2 ? 0 : q3L + 1;
             const int gkLm = gkLc, gkGm = gkGc, gkUm = gkUc;
-            const int sLr = NRING == 4 ? (kL & 3) : q3L, sGr = NRING == 4 ? (kG & 3) : q3G, sUr = NRING == 4 ? (kU & 3) : q3U;
+            const int sLr = q3L, sGr = q3G, sUr = q3U;
             const bool do_grad = kG >= k0 - 1 && kG <= k1 && !(!pk && kG == 0);
             // the first plane of a non-periodic k axis: formed with plane 1
             const bool do_grad0 = !pk && kG == 1 && k0 == 1;
@@ -1021,9 +769,6 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                     S.PH[cell] = add2(e, p);
                 }
             }
-            // separable form: thread 0's spacing copy of plane kL - 1 (issued
-            // two iterations ago) has landed, and the barrier publishes it
-            if (SEP && tid == 0) cp_async_wait_prev();
             // (a thread whose staging wait gave up turns staging off for the
             // whole CTA here)
             tma_off = __syncthreads_or(tma_off) != 0;
@@ -1034,13 +779,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             // plane (kL), waited for in the next iteration, and Q(0) of this
             // iteration's updated points (plane kL - 2), waited for before
             // the update; each thread copies, and later reads, its own values
-            if constexpr (!SEP) {
-                if (kL >= k0 - 1 && kL <= k1) fetch_met(gkLm, q3L);
-            } else {
-                // the spacings of plane kL + 1 into the slot of plane kL - 3,
-                // whose last reads preceded the barrier above
-                if (tid == 0) cp_async16(S.HZ + ((kL + 1) & 3), F.h1[2] + map_idx(kL + 1, nk, pk));
-            }
+            if (kL >= k0 - 1 && kL <= k1) fetch_met(gkLm, q3L);
             if (!rhs_only && kL - 2 >= k0 && kL - 2 <= k1 - 1) {
                 const int pU = gkUm * plane;
                 const float *Q0 = J.q[0];
@@ -1060,7 +799,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             // chunk's first zeta interface
             if (kL == k0) wof(CK_RING(sUr * N2 + c2), Wc);
             // ---- gradients of plane kG (and of plane 0, late) ----
-            if (!SEP && (do_grad || do_grad0)) cp_async_wait_prev();
+            if (do_grad || do_grad0) cp_async_wait_prev();
             if (do_grad0) grad(0, map_idx(0, nk, pk), r3(0), r3(-1), r3(1));
             if (do_grad) grad(kG, gkGm, q3G, q3U, q3L);
             // ---- interfaces and update of plane kU ----
@@ -1075,19 +814,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                 float2 WL[5];
                 wvec(L, WL);
                 float2 mL[9], jL = bc(0.0f);
-                if constexpr (!SEP) mets(mU, c1, mL, jL);
-                // separable form: spacings of the own points and their neighbours
-                float4 hXo = make_float4(0.f, 0.f, 0.f, 0.f), hXp = hXo, hZo = hXo, hZp = hXo;
-                float2 hYo = bc(0.f), rhYo = bc(0.f);
-                if constexpr (SEP) {
-                    hXo = S.HX[tx + 1];
-                    hXp = S.HX[tx + 2];
-                    hZo = S.HZ[kU & 3];
-                    hZp = S.HZ[(kU + 1) & 3];
-                    const float4 yA = S.HY[rA + 2], yB = S.HY[rB + 2];
-                    hYo = f2(yA.x, yB.x);
-                    rhYo = f2(yA.y, yB.y);
-                }
+                mets(mU, c1, mL, jL);
                 float2 hx[5], hy[5], hz[5];
 #pragma unroll
                 for (int f = 0; f < 5; ++f) {
@@ -1116,16 +843,9 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                     Side SL, SR;
                     side(2, rU, c1, SL);
                     side(2, rP, c1, SR);
-                    if constexpr (SEP) {
-                        const float2 Sa = mul2(bc(hXo.x), hYo);
-                        const float2 hb = bc(0.5f * (hZo.x + hZp.x));
-                        iface_sep<2>(FP, L, WL, R, WR, Wc, WRp, SL, SR, Sa, hb, rcp2(hb), bc(0.25f * hXo.y),
-                                     mul2(bc(0.25f), rhYo), hz);
-                    } else {
-                        float2 mR[9], jR;
-                        mets(mP, c1, mR, jR);
-                        iface<2>(FP, L, WL, mL, jL, R, WR, mR, jR, Wc, WRp, SL, SR, hz);
-                    }
+                    float2 mR[9], jR;
+                    mets(mP, c1, mR, jR);
+                    iface<2>(FP, L, WL, mL, jL, R, WR, mR, jR, Wc, WRp, SL, SR, hz);
                 };
                 if (!first) {
                     // eta: R = (own second row, first row of the pair cell
@@ -1154,22 +874,13 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                         for (int b = 0; b < 2; ++b)
 #pragma unroll
                             for (int f = 0; f < 4; ++f) SR.d[b][f] = odd2(SL.d[b][f], SU.d[b][f]);
-                        if constexpr (SEP) {
-                            const float4 yC = S.HY[rB + 3]; // row 2tr+2
-                            const float2 hYR = f2(hYo.y, yC.x);
-                            const float2 Sa = bc(hXo.x * hZo.x);
-                            const float2 hb = mul2(bc(0.5f), add2(hYo, hYR));
-                            iface_sep<1>(FP, L, WL, R, WR, WLm, WP1, SL, SR, Sa, hb, rcp2(hb), bc(0.25f * hXo.y),
-                                         bc(0.25f * hZo.y), hy);
-                        } else {
-                            float2 mA[9], jA, mR[9];
-                            mets(mU, up, mA, jA);
+                        float2 mA[9], jA, mR[9];
+                        mets(mU, up, mA, jA);
 #pragma unroll
-                            for (int t = 0; t < 9; ++t) mR[t] = odd2(mL[t], mA[t]);
-                            iface<1>(FP, L, WL, mL, jL, R, WR, mR, odd2(jL, jA), WLm, WP1, SL, SR, hy);
-                        }
+                        for (int t = 0; t < 9; ++t) mR[t] = odd2(mL[t], mA[t]);
+                        iface<1>(FP, L, WL, mL, jL, R, WR, mR, odd2(jL, jA), WLm, WP1, SL, SR, hy);
                     }
-                    if constexpr (!SEP) zeta();
+                    zeta();
                     // xi: R = the next column.  Lane 31's R has no R1 data: it pairs
                     // with its own R1 cell (an unused result), so that every lane
                     // runs the xi flux without a branch and the scheduler can
@@ -1184,24 +895,15 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                         Side SL, SR;
                         side(0, rU, c1, SL);
                         side(0, rU, cR, SR);
-                        if constexpr (SEP) {
-                            // Sa = h_y h_z, hb = average h_x, tangential 1/(4 h)
-                            const float2 Sa = mul2(hYo, bc(hZo.x));
-                            const float2 hb = bc(0.5f * (hXo.x + hXp.x));
-                            iface_sep<0>(FP, L, WL, R, WR, WLm, WRp, SL, SR, Sa, hb, rcp2(hb),
-                                         mul2(bc(0.25f), rhYo), bc(0.25f * hZo.y), hx);
-                        } else {
-                            float2 mR[9], jR;
-                            mets(mU, cR, mR, jR);
-                            iface<0>(FP, L, WL, mL, jL, R, WR, mR, jR, WLm, WRp, SL, SR, hx);
-                        }
+                        float2 mR[9], jR;
+                        mets(mU, cR, mR, jR);
+                        iface<0>(FP, L, WL, mL, jL, R, WR, mR, jR, WLm, WRp, SL, SR, hx);
                     }
 #pragma unroll
                     for (int f = 0; f < 5; ++f) S.SH[CK_SH(f * NT + tid)] = hy[f].y;
-                } else if constexpr (!SEP) {
+                } else {
                     zeta();
                 }
-                if constexpr (SEP) zeta();
                 // the -1/2 xi flux from the lane below (all lanes of the warp
                 // take part in the shuffle; the CTA-uniform `first` guards it)
                 float2 hxm[5];
@@ -1255,7 +957,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                     hz_prev[f] = hz[f];
                     Wc[f] = WL[f];
                 }
-            } else if (NRING == 3) {
+            } else {
                 __syncthreads(); // as in the branch above: this iteration's ring reads
                                  // precede the next iteration's loads into the freed slot
             }
@@ -1323,31 +1025,19 @@ void launch_pack_pairs(const float *met, long long fs, int pitch, int nj, int nk
 
 template <int TY> int fused_prepare()
 {
-    int rc = (int)cudaFuncSetAttribute(k_fused<TY, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Geo<TY, false>::BYTES);
-    if (!rc) rc = (int)cudaFuncSetAttribute(k_fused<TY, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)Geo<TY, true>::BYTES);
-    if (!rc) rc = (int)cudaFuncSetAttribute(k_fused<TY, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)Geo<TY, false>::BYTES);
-    if (!rc) rc = (int)cudaFuncSetAttribute(k_fused<TY, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)Geo<TY, true>::BYTES);
+    int rc = (int)cudaFuncSetAttribute(k_fused<TY, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)Geo<TY>::BYTES);
+    if (!rc) rc = (int)cudaFuncSetAttribute(k_fused<TY, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)Geo<TY>::BYTES);
     return rc;
 }
 
-int fused_ctas_per_sm(int ty, int separable)
+int fused_ctas_per_sm(int ty)
 {
     int n = 0;
-    cudaError_t e;
-    if (ty == 16)
-        e = separable ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<16, true, true>, FX * 8,
-                                                                      Geo<16, true>::BYTES)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<16, false, true>, FX * 8,
-                                                                      Geo<16, false>::BYTES);
-    else
-        e = separable ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<8, true, true>, FX * 4,
-                                                                      Geo<8, true>::BYTES)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<8, false, true>, FX * 4,
-                                                                      Geo<8, false>::BYTES);
+    const cudaError_t e =
+        ty == 16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<16, true>, FX * 8, Geo<16>::BYTES)
+                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_fused<8, true>, FX * 4, Geo<8>::BYTES);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -1356,41 +1046,29 @@ int fused_ctas_per_sm(int ty, int separable)
 }
 
 template <int TY>
-void launch_fused(const JetDev<float> *jets, const FusedJet *fj, int njets, int total_items, int total_tiles,
-                  int grid, int src, int dst, int stage, const double *dt, int rhs_only, int separable, int balanced,
-                  int wait_limit, const JetDev<float> *j1, const FusedJet *f1, cudaStream_t st)
+static void launch_one(const FusedLaunch &a, int grid, const JetDev<float> &ja, const FusedJet &fa, bool one, cudaStream_t st)
 {
-    dim3 block(FX, TY / 2);
-    if (wait_limit < 0) wait_limit = MBAR_WAIT_LIMIT;
-    const bool one = njets == 1 && j1 && f1;
-    JetDev<float> jz{};
-    FusedJet fz{};
+    const dim3 block(FX, TY / 2);
+    const int lim = a.wait_limit < 0 ? MBAR_WAIT_LIMIT : a.wait_limit;
+    if (one)
+        k_fused<TY, true><<<grid, block, Geo<TY>::BYTES, st>>>(a.jets, a.fj, a.njets, a.items, a.tiles, a.src, a.dst,
+                                                              a.stage, a.dt, a.rhs_only, a.balanced, lim, ja, fa);
+    else
+        k_fused<TY, false><<<grid, block, Geo<TY>::BYTES, st>>>(a.jets, a.fj, a.njets, a.items, a.tiles, a.src, a.dst,
+                                                               a.stage, a.dt, a.rhs_only, a.balanced, lim, ja, fa);
+}
+void launch_fused(int ty, const FusedLaunch &a, int grid, const JetDev<float> *j1, const FusedJet *f1, cudaStream_t st)
+{
+    const bool one = a.njets == 1 && j1 && f1;
+    static const JetDev<float> jz{};
+    static const FusedJet fz{};
     const JetDev<float> &ja = one ? *j1 : jz;
     const FusedJet &fa = one ? *f1 : fz;
-    if (separable) {
-        if (one)
-            k_fused<TY, true, true><<<grid, block, Geo<TY, true>::BYTES, st>>>(
-                jets, fj, njets, total_items, total_tiles, src, dst, stage, dt, rhs_only, balanced, wait_limit, ja, fa);
-        else
-            k_fused<TY, true, false><<<grid, block, Geo<TY, true>::BYTES, st>>>(
-                jets, fj, njets, total_items, total_tiles, src, dst, stage, dt, rhs_only, balanced, wait_limit, ja, fa);
-    } else {
-        if (one)
-            k_fused<TY, false, true><<<grid, block, Geo<TY, false>::BYTES, st>>>(
-                jets, fj, njets, total_items, total_tiles, src, dst, stage, dt, rhs_only, balanced, wait_limit, ja, fa);
-        else
-            k_fused<TY, false, false><<<grid, block, Geo<TY, false>::BYTES, st>>>(
-                jets, fj, njets, total_items, total_tiles, src, dst, stage, dt, rhs_only, balanced, wait_limit, ja, fa);
-    }
+    if (ty == 16) launch_one<16>(a, grid, ja, fa, one, st);
+    else launch_one<8>(a, grid, ja, fa, one, st);
 }
 
 template int fused_prepare<16>();
 template int fused_prepare<8>();
-template void launch_fused<16>(const JetDev<float> *, const FusedJet *, int, int, int, int, int, int, int,
-                               const double *, int, int, int, int, const JetDev<float> *, const FusedJet *,
-                               cudaStream_t);
-template void launch_fused<8>(const JetDev<float> *, const FusedJet *, int, int, int, int, int, int, int,
-                              const double *, int, int, int, int, const JetDev<float> *, const FusedJet *,
-                              cudaStream_t);
 
 } // namespace les

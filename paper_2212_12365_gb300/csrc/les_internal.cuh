@@ -283,17 +283,29 @@ constexpr int tma_box_rows(int ty) { return ty + 4; }
 void set_call_error(const char *msg);
 
 template <int TY> int fused_prepare();
-// resident CTAs per SM of the fused stage for tile height ty (general or
-// separable form), from the occupancy calculator; 1 if it cannot tell
-int fused_ctas_per_sm(int ty, int separable);
-// One launch of the fused stage.  jets / fj: the device tables of the njets
-// jets; for a single jet (njets == 1) j1 / f1 are host copies of its two
-// entries, passed by value as kernel parameters, so that the kernel reads the
-// jet's constants from the parameter bank (null otherwise).
-template <int TY>
-void launch_fused(const JetDev<float> *jets, const FusedJet *fj, int njets, int total_items, int total_tiles,
-                  int grid, int src, int dst, int stage, const double *dt, int rhs_only, int separable, int balanced,
-                  int wait_limit, const JetDev<float> *j1, const FusedJet *f1, cudaStream_t st);
+// resident CTAs per SM of the general form at tile height ty, from the
+// occupancy calculator; 1 if it cannot tell
+int fused_ctas_per_sm(int ty);
+
+// Arguments of one launch of the fused FP32 stage: the device tables of the
+// njets jets, and the work list.
+struct FusedLaunch {
+    const JetDev<float> *jets;
+    const FusedJet *fj;
+    int njets, items, tiles, src, dst, stage;
+    const double *dt;
+    int rhs_only, balanced, wait_limit;
+};
+// One launch of the general form (les_fused.cu; ty 8 or 16).  For a single jet
+// (njets == 1) j1 / f1 are host copies of its two table entries, passed by
+// value as kernel parameters, so that the kernel reads the jet's constants
+// from the parameter bank (null otherwise).
+void launch_fused(int ty, const FusedLaunch &a, int grid, const JetDev<float> *j1, const FusedJet *f1, cudaStream_t st);
+// The product-grid form (les_fused_prod.cu; ty 8, 16 or 24).
+int fused_prod_prepare();
+int fused_prod_ctas_per_sm(int ty);
+void launch_fused_prod(int ty, const FusedLaunch &a, int grid, const JetDev<float> *j1, const FusedJet *f1,
+                       cudaStream_t st);
 
 // General FP32 form: the paired static records (see FusedJet::mp) from the
 // FP32 static fields; mp holds nk * ((nj + 1) / 2) * 5 * pitch float4.
