@@ -299,7 +299,7 @@ int les_bounds_violation(les_handle *h, uint64_t *out);
  *               [11] count of non-finite values;
  *   stream    : cudaStream_t the two kernels are launched on (NULL allowed).
  * Asynchronous; allocates nothing.  Its scratch is one file-scope device
- * array of 608 x 17 doubles (83 KB), held by every
+ * array of 304 x 17 doubles (41 KB), held by every
  * GPU that loads the library until exit; the first call on a device looks up
  * that array's device address (make it before any stream capture).  All calls
  * share the array: calls that overlap on the GPU (different streams without

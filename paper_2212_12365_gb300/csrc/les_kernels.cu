@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(BLOCK) k_dt_max(const JetDev<real> *__restrict
 // ---------------------------------------------------------------------------
 
 template <typename real>
-__global__ void __launch_bounds__(SUM_BLOCK, 4) k_diag_partials(const JetDev<real> *__restrict__ jets,
+__global__ void __launch_bounds__(SUM_BLOCK, SUM_BLOCKS_PER_SM) k_diag_partials(const JetDev<real> *__restrict__ jets,
                                                                 int jet, double *part)
 {
     const JetDev<real> &J = jets[jet];

@@ -12,7 +12,7 @@
 // truncated tails are below 2^-96 of the largest value each, so the sum is as
 // good as the compensated one (a test holds both to the exactly rounded sum).
 // The sums of squares stay in FP64 (one multiply-add per value).
-// Measured: 14,155,776 points 2098 -> 319 us (3.5 TB/s); les_get_diagnostics of
+// Measured: 14,155,776 points 2098 -> 236 us (4.8 TB/s); les_get_diagnostics of
 // a 192x128x72 FP32 jet about 1.0 ms less per call (most of it the final pass).
 #pragma once
 
@@ -24,7 +24,11 @@ constexpr int SUM_PART = 17;      // partial results per block, field-major [f][
                                   // 0 max |RHS_rho|, 1..5 sum RHS^2, 6..10 sum Qhat,
                                   // 11..15 its compensation, 16 non-finite count
 constexpr int SUM_BLOCK = 256;    // threads per block
-constexpr int SUM_MAX_BLOCKS = 608; // 4 blocks on each of 152 SMs: one wave, 32 warps per SM
+// One wave: two blocks on each of 152 SMs, whose threads keep the next point's
+// ten values in flight in registers (123 of them).  Four blocks without that
+// read-ahead took 319 us at 14,155,776 points, three with it 287 (spills), two 250.
+constexpr int SUM_BLOCKS_PER_SM = 2;
+constexpr int SUM_MAX_BLOCKS = 152 * SUM_BLOCKS_PER_SM;
 
 __device__ __forceinline__ void neumaier_add(double &s, double &c, double v)
 {
@@ -111,13 +115,22 @@ struct SumFx {
 template <typename Load> __device__ __forceinline__ void sum_block(long long steps, const Load &load, double *part)
 {
     SumFx fx[5];
-    double mx = 0.0, l2[5] = {0, 0, 0, 0, 0};
+    double l2[5] = {0, 0, 0, 0, 0};
+    long long mxb = 0; // |RHS_rho| as its bits, which order as integers (NaN ignored, as fmax does)
     int bad = 0;
     unsigned nf = 0; // fields that met a non-finite value: their sum is NaN
+    double qn[5], rn[5];
+    load(0, qn, rn);
     for (long long t = 0; t < steps; ++t) {
         double q[5], r[5];
-        load(t, q, r);
-        mx = fmax(mx, fabs(r[0]));
+#pragma unroll
+        for (int f = 0; f < 5; ++f) {
+            q[f] = qn[f];
+            r[f] = rn[f];
+        }
+        if (t + 1 < steps) load(t + 1, qn, rn); // in flight while this point is added
+        const long long ab = __double_as_longlong(r[0]) & 0x7fffffffffffffffll;
+        mxb = max(mxb, ab > 0x7ff0000000000000ll ? 0ll : ab);
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
             const bool vf = (((unsigned)__double2hiint(q[f]) >> 20) & 0x7ffu) != 0x7ffu;
@@ -130,6 +143,7 @@ template <typename Load> __device__ __forceinline__ void sum_block(long long ste
     }
     __shared__ double sh[SUM_PART][SUM_BLOCK / 32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double mx = __longlong_as_double(mxb);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -180,7 +194,7 @@ inline int sum_blocks(long long n)
 
 // Combine nb blocks' partials into out[12] (see les_diag_sums_noalloc); a
 // warp per result, lanes over the blocks, then a fixed shuffle tree.  (One
-// thread walking the 17 x nb values in turn took 0.25 ms at 608 blocks.)
+// thread walking 17 x 608 values in turn took 0.25 ms.)
 constexpr int SUM_FINAL_THREADS = 12 * 32;
 __device__ __forceinline__ void sum_final(const double *__restrict__ part, int nb, double *out)
 {
