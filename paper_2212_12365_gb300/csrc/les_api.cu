@@ -99,7 +99,8 @@ struct les_handle {
         int cps[3] = {1, 1, 1};         // resident CTAs per SM at tile height 8, 16, 24
         std::string note;
     } form[2];
-    std::vector<JetDev<float>> jd32;    // host copy of the FP32 jet table
+    std::vector<JetDev<float>> jd32;    // host copy of the jet table (FP32, FP64 handles)
+    std::vector<JetDev<double>> jd64;
     bool tuned = false;
     int64_t launches_per_step = 0;
     int64_t last_launches = 0;
@@ -369,7 +370,20 @@ template <typename real> static void fill_jetdev(const les_handle *h, const JetH
     D.bc_rg = 1.0 / p.gamma;
     D.bc_cinf = std::sqrt(p.gamma * (1.0 / p.gamma) / p.TR);
     D.seed = (unsigned long long)p.seed;
-    (void)h;
+    auto pair = [](double v, float &hi, float &lo) {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    };
+    D.bcf.g = (float)p.gamma;
+    D.bcf.g1 = (float)D.bc_g1;
+    D.bcf.rg = (float)D.bc_rg;
+    D.bcf.TR = (float)p.TR;
+    D.bcf.cinf = (float)D.bc_cinf;
+    D.bcf.e2 = (float)(2.0 * D.bc_g1);
+    D.bcf.e2g = (float)(2.0 * p.gamma * D.bc_g1);
+    pair(p.gamma - 1.0, D.bcf.gm1h, D.bcf.gm1l);
+    pair(p.gamma * (p.gamma - 1.0), D.bcf.ggm1h, D.bcf.ggm1l);
+    pair(1.0 / p.TR, D.bcf.Tinfh, D.bcf.Tinfl);
 }
 
 template <typename real> static int setup_jet(les_handle *h, JetHost &J, const les_grid_desc *g)
@@ -706,6 +720,7 @@ static int create_impl(const les_grid_desc *g, const les_params *p, int njets, v
     for (int j = 0; j < njets; ++j) fill_jetdev<real>(h, h->J[j], D[j]);
     CK(cudaMemcpyAsync(h->d_jets, D.data(), sizeof(JetDev<real>) * njets, cudaMemcpyHostToDevice, h->st));
     if constexpr (sizeof(real) == sizeof(float)) h->jd32 = D;
+    else h->jd64 = D;
     if (h->prec == LES_FP32) {
         if (fused_prepare<16>() != 0 || fused_prepare<8>() != 0 || fused_prod_prepare() != 0)
             return bail(fail(h, LES_ERR_CUDA, "fused kernel shared-memory attribute"));
@@ -844,33 +859,45 @@ extern "C" int les_create_batch(const les_grid_desc *g, const les_params *p, int
 
 static int grid_cap(les_handle *h, int total) { return std::max(1, std::min(total, h->nsm * 8)); }
 
-// One part (0 point, 1 gradients, 2 interfaces, 3 update) of the FP64 stage:
-// the jets of the general form (map g), then those of the product form (map
-// p); returns the number of launches.
-static int fp64_part(les_handle *h, const JetDev<double> *jets, const BlockMap &g, const BlockMap &p, int part, int src,
-                     int dst, int stage, int rhs_only, cudaStream_t st)
+// Host copy of the table entry of the only jet of a launch over jets (all of
+// them, jet < 0, or one); null if there are several.
+template <typename real> static const JetDev<real> *only_jet(const les_handle *h, int jet)
 {
+    if (jet < 0 && h->njets > 1) return nullptr;
+    if constexpr (sizeof(real) == sizeof(float)) return &h->jd32[jet < 0 ? 0 : jet];
+    else return &h->jd64[jet < 0 ? 0 : jet];
+}
+
+// One part (0 point, 1 gradients, 2 interfaces, 3 update) of the FP64 stage over
+// all jets (jet < 0) or one: the jets of the general form, then those of the
+// product form.  Returns the number of launches.
+static int fp64_part(les_handle *h, int jet, int part, int src, int dst, int stage, int rhs_only, cudaStream_t st)
+{
+    const JetDev<double> *jets = (const JetDev<double> *)h->d_jets + (jet < 0 ? 0 : jet);
+    const BlockMap &g = jet < 0 ? h->ptg : h->ptg1[jet], &p = jet < 0 ? h->ptp : h->ptp1[jet];
+    const double *dt = h->d_dt + (jet < 0 ? 0 : jet);
     if (g.total > 0) {
         const int gp = grid_cap(h, g.total);
         switch (part) {
         case 0: Launch<double>::point(jets, g, src, gp, st); break;
         case 1: Launch<double>::grads(jets, g, gp, st); break;
         case 2: Launch<double>::iface(jets, g, gp, st); break;
-        default: Launch<double>::update(jets, g, dst, stage, h->d_dt, rhs_only, gp, st); break;
+        default: Launch<double>::update(jets, g, dst, stage, dt, rhs_only, gp, st); break;
         }
     }
     // one block per 64 points: the hardware balances them over the SMs
-    if (p.total > 0) launch_stage_prod(jets, p, part, src, dst, stage, h->d_dt, rhs_only, p.total, st);
+    if (p.total > 0) launch_stage_prod(jets, p, part, src, dst, stage, dt, rhs_only, p.total, st);
     return (g.total > 0) + (p.total > 0);
 }
 
-// Boundary conditions of the current level on the jets of the map; returns the
-// number of launches.
-template <typename real>
-static int bc_pass(les_handle *h, const BlockMap &bm, const JetDev<real> *jets, int dst, cudaStream_t st)
+// Boundary conditions of the current level on all jets (jet < 0) or one;
+// returns the number of launches.
+template <typename real> static int bc_pass(les_handle *h, int jet, int dst, cudaStream_t st)
 {
+    const JetDev<real> *jets = (const JetDev<real> *)h->d_jets + (jet < 0 ? 0 : jet);
+    const BlockMap &bm = jet < 0 ? h->bcm : h->bc1[jet];
     if (h->centerline) launch_centerline<real>(jets, bm.njets, h->max_ni, dst, st);
-    Launch<real>::bc(jets, bm, dst, h->d_level, st);
+    Launch<real>::bc(jets, bm, dst, h->d_level, only_jet<real>(h, jet), st);
     return (h->centerline ? 1 : 0) + (bm.total > 0 ? 1 : 0);
 }
 
@@ -915,20 +942,19 @@ template <typename real> static int record_step(les_handle *h, cudaStream_t st, 
             T.end();
             if (h->bcm.total > 0) { // none on a fully periodic grid
                 T.begin(LES_KERNEL_BC);
-                h->launches_per_step += bc_pass<real>(h, h->bcm, jets, dst_of[s], st);
+                h->launches_per_step += bc_pass<real>(h, -1, dst_of[s], st);
                 T.end();
             }
             continue;
         }
         for (int part = 0; part < 4; ++part) {
             T.begin(LES_KERNEL_POINT + part);
-            h->launches_per_step += fp64_part(h, (const JetDev<double> *)h->d_jets, h->ptg, h->ptp, part, src_of[s],
-                                              dst_of[s], s, 0, st);
+            h->launches_per_step += fp64_part(h, -1, part, src_of[s], dst_of[s], s, 0, st);
             T.end();
         }
         if (h->bcm.total > 0) { // none on a fully periodic grid
             T.begin(LES_KERNEL_BC);
-            h->launches_per_step += bc_pass<real>(h, h->bcm, jets, dst_of[s], st);
+            h->launches_per_step += bc_pass<real>(h, -1, dst_of[s], st);
             T.end();
         }
     }
@@ -1039,7 +1065,7 @@ template <typename real> static int set_state_impl(les_handle *h, int jet, const
     CK(cudaGetLastError());
     // boundary conditions of the current level on this jet (faces y, z, x)
     const JetDev<real> *one = jets + jet;
-    bc_pass<real>(h, h->bc1[jet], one, 0, h->st);
+    bc_pass<real>(h, jet, 0, h->st);
     CK(cudaGetLastError());
     if (h->dt[jet] == 0.0) {
         BlockMap p1 = h->pt1[jet];
@@ -1123,8 +1149,7 @@ template <typename real> static int residual_of_jet(les_handle *h, int jet)
         CK(cudaGetLastError());
         return LES_OK;
     }
-    for (int part = 0; part < 4; ++part)
-        fp64_part(h, (const JetDev<double> *)h->d_jets + jet, h->ptg1[jet], h->ptp1[jet], part, 0, 0, 0, 1, h->st);
+    for (int part = 0; part < 4; ++part) fp64_part(h, jet, part, 0, 0, 0, 1, h->st);
     CK(cudaGetLastError());
     return LES_OK;
 }

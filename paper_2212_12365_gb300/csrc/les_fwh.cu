@@ -29,6 +29,7 @@
 
 #include "les_fp64.cuh"
 #include "les_internal.cuh"
+#include "les_pair.cuh"
 
 namespace les {
 
@@ -74,51 +75,6 @@ __device__ __forceinline__ void store8(float4 *p, const float4 &a, const float4 
 // FP32, so both give the same records up to rare ties, and the pairs run on the
 // FP32 pipe, 64 times as wide as the FP64 pipe that bounded this pass (98,304
 // panels x 1024 frames: 7.6 -> 1.3 ms; now 3.7 TB/s of reads and writes).
-template <typename real> struct Num;
-template <> struct Num<double> {
-    typedef double T;
-    static __device__ __forceinline__ T of(double v) { return v; }
-    static __device__ __forceinline__ T mul(double a, T b) { return a * b; }
-    static __device__ __forceinline__ T mulp(T a, T b) { return a * b; }
-    static __device__ __forceinline__ T add(T a, T b) { return a + b; }
-    static __device__ __forceinline__ T sub(T a, T b) { return a - b; }
-    static __device__ __forceinline__ float out(T a) { return (float)a; }
-};
-struct FloatPair {
-    float h, l;
-};
-template <> struct Num<float> {
-    typedef FloatPair T;
-    static __device__ __forceinline__ T of(double v)
-    {
-        const float h = (float)v;
-        return {h, (float)(v - (double)h)};
-    }
-    static __device__ __forceinline__ T quick(float a, float b) // |a| >= |b|
-    {
-        const float s = __fadd_rn(a, b);
-        return {s, __fsub_rn(b, __fsub_rn(s, a))};
-    }
-    static __device__ __forceinline__ T mul(float a, T b)
-    {
-        const float p = __fmul_rn(a, b.h);
-        return quick(p, __fmaf_rn(a, b.l, __fmaf_rn(a, b.h, -p)));
-    }
-    static __device__ __forceinline__ T mulp(T a, T b)
-    {
-        const float p = __fmul_rn(a.h, b.h);
-        return quick(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
-    }
-    static __device__ __forceinline__ T add(T a, T b)
-    {
-        const float s = __fadd_rn(a.h, b.h), v = __fsub_rn(s, a.h);
-        const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, v)), __fsub_rn(b.h, v));
-        return quick(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
-    }
-    static __device__ __forceinline__ T sub(T a, T b) { return add(a, T{-b.h, -b.l}); }
-    static __device__ __forceinline__ float out(T a) { return __fadd_rn(a.h, a.l); }
-};
-
 // Per (panel j of the batch, frame m): src[(j*N + m)*2] = (L_x, L_y, L_z,
 // dQ/dtau), src[(j*N + m)*2 + 1] = (dL_x/dtau, dL_y/dtau, dL_z/dtau, 0).  One
 // thread per panel and segment of SEG frames marches its frames with the

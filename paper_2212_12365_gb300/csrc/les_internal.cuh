@@ -65,6 +65,14 @@ enum { PT_H = 0, PT_RH, PT_RH4, PT_RH6, PT_HB, PT_RHB, PT_RHB43, PROD_TABS };
 constexpr int DBG_RHS = 100;  // debug export codes beside the LES_FIELD_* values
 constexpr int DBG_MET0 = 200;
 
+// Constants of the FP32 boundary arithmetic: gamma, 1/(gamma-1), 1/gamma,
+// ambient density and speed of sound, 2/(gamma-1), 2 gamma/(gamma-1); as pairs
+// of floats gamma - 1, gamma (gamma - 1) and the ambient T = 1/TR.
+struct BcConst {
+    float g, g1, rg, TR, cinf, e2, e2g;
+    float gm1h, gm1l, ggm1h, ggm1l, Tinfh, Tinfl;
+};
+
 // Geometry and parameters of one jet, as seen by the kernels.
 template <typename real>
 struct JetDev {
@@ -91,6 +99,7 @@ struct JetDev {
     double kap_mol;    // mu -> conductivity: 1/(Re Pr (gamma-1))
     double kap_sgs;    // mu_sgs -> conductivity: 1/(Pr_sgs (gamma-1))
     double bc_g1, bc_rg, bc_cinf; // 1/(gamma-1), 1/gamma, ambient sound speed (1/TR)^1/2
+    BcConst bcf;
     unsigned long long seed;
     long long npts_pad; // nk*nj*pitch
     // first out-of-range index met by a kernel of a LES_BOUNDS_CHECK build
@@ -338,7 +347,9 @@ template <typename real> struct Launch {
     static void iface(const JetDev<real> *jets, BlockMap bm, int grid, cudaStream_t st);
     static void update(const JetDev<real> *jets, BlockMap bm, int dst, int stage,
                        const double *dt, int rhs_only, int grid, cudaStream_t st);
-    static void bc(const JetDev<real> *jets, BlockMap bm, int dst, const long long *level, cudaStream_t st);
+    // j1: host copy of a single jet's table entry, passed by value (see launch_fused), or null
+    static void bc(const JetDev<real> *jets, BlockMap bm, int dst, const long long *level, const JetDev<real> *j1,
+                   cudaStream_t st);
     static void set_state(const JetDev<real> *jets, int jet, const double *in, int kind,
                           long long npad, cudaStream_t st);
     static void get_state(const JetDev<real> *jets, int jet, double *out, int kind,
