@@ -48,17 +48,19 @@ __device__ __forceinline__ double rsqrt64(double x)
     return fma(y, e * fma(0.375, e, 0.5), y);
 }
 // x^1/2, x >= 0; 0 below the normal range
-__device__ __forceinline__ double sqrt64_scaled(double x, int twice)
+template <int E> // times 2^E
+__device__ __forceinline__ double sqrt64_scaled(double x)
 {
     const double y = rsqrt_seed64(x);
     const double t0 = x * y;
     const double e = fma(-t0, y, 1.0);
-    const double t = twice ? __hiloint2double(__double2hiint(t0) + (1 << 20), __double2loint(t0)) : t0;
+    const double t = E != 0 ? __hiloint2double(__double2hiint(t0) + E * (1 << 20), __double2loint(t0)) : t0;
     const double s = fma(t, e * fma(0.375, e, 0.5), t);
     return __double2hiint(x) < 0x00100000 && __double2hiint(x) >= 0 ? 0.0 : s;
 }
-__device__ __forceinline__ double sqrt64(double x) { return sqrt64_scaled(x, 0); }
-__device__ __forceinline__ double twice_sqrt64(double x) { return sqrt64_scaled(x, 1); }
+__device__ __forceinline__ double sqrt64(double x) { return sqrt64_scaled<0>(x); }
+__device__ __forceinline__ double twice_sqrt64(double x) { return sqrt64_scaled<1>(x); }
+__device__ __forceinline__ double half_sqrt64(double x) { return sqrt64_scaled<-1>(x); }
 // max of two non-negative numbers (their bit patterns order as integers)
 __device__ __forceinline__ double max_nn(double a, double b)
 {

@@ -32,9 +32,9 @@ constexpr int MET_RJB = 15;   // + a
 constexpr int MET_NORM = 18;  // + a
 // FP64 only, per axis a at [MET_A0 + 9a + 3b + c]: the interface (to the +a
 // neighbour) average of the cofactor J^-1 d xi^b / d x_c divided by the
-// interface J^-1, times 1/2 for b != a: the chain-rule weights of the compact
+// interface J^-1, times 1/4 for b != a: the chain-rule weights of the compact
 // viscous flux applied to the normal difference (b == a) and to the SUM of
-// the two points' central differences (b != a).
+// the two points' doubled central differences (b != a).
 // FP64 only, per axis a at [MET_K0 + 3a + b]: K_b = sum_c A_ac A_bc (same
 // tables), so that the flux-direction contraction of a gradient,
 // sum_c A_ac d phi/d x_c, is sum_b K_b D_b.
@@ -46,7 +46,7 @@ enum {
     P_RHO = 0, P_U, P_V, P_W, P_P, P_T, P_MU, P_LXI, P_LETA, P_LZETA,
     P_RU, P_RV, P_RW, P_RH, P_F0
 };
-// Per-point derivative fields: d(u,v,w,T)/d(xi,eta,zeta) at [3*phi + axis],
+// Per-point derivative fields: 2 d(u,v,w,T)/d(xi,eta,zeta) at [3*phi + axis],
 // mu_sgs, mu/Re + mu_sgs, the total conductivity, and the pressure sensor
 // per axis.
 constexpr int NGRAD = 18;

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(BLOCK) k_static_fields(double *met, long long 
                 for (int b = 0; b < 3; ++b)
                     for (int c = 0; c < 3; ++c) {
                         const double mc = 0.5 * (met[(3 * b + c) * fs + o] + met[(3 * b + c) * fs + oR]);
-                        A[3 * b + c] = mc * rjb * (b == a ? 1.0 : 0.5);
+                        A[3 * b + c] = mc * rjb * (b == a ? 1.0 : 0.25);
                         met[(MET_A0 + 9 * a + 3 * b + c) * fs + o] = A[3 * b + c];
                     }
                 for (int b = 0; b < 3; ++b)

@@ -20,47 +20,36 @@
 // direction telescopes exactly.  On GB300 the FP64 form is bound by the FP64
 // pipe, not by HBM: the intermediate fields cost bandwidth that is otherwise
 // idle and remove recomputation (divisions, square roots) from the hot loop.
+// Jets on a Cartesian-product grid take les_stage_prod.cu; this is the form for
+// curvilinear ones.  Measured on the 200x75x40 polar mesh, us per launch, with
+// the short root and reciprocal sequences, integer maxima and doubled
+// differences: point 135 -> 120, gradients 134 -> 108, interfaces 403 -> 396.
 #include <cmath>
 
+#include "les_fp64.cuh"
 #include "les_internal.cuh"
 
 namespace les {
 
 __constant__ double c_alpha[5] = {0.25, 1.0 / 6.0, 0.375, 0.5, 1.0};
 
-// Reciprocal.  FP32 uses the hardware division.  In FP64, whose pipe is the
-// bottleneck on this GPU, the reciprocal is a Newton-Raphson iteration
-// r <- r (2 - b r) from the hardware's approximate FP64 reciprocal (a seed of
-// about single precision, taken without converting through FP32): each step
-// squares the relative error, so two steps reach double rounding (a unit in
-// the last place) at fewer FP64 operations than an IEEE division, and one
-// step leaves a relative error near 1e-14, which is all a factor needs whose
-// own error enters the residual damped by its small weight (pressure sensor,
-// Sutherland law).  Arguments are positive normal numbers (densities,
-// temperatures, sensor denominators).  Square roots stay the native ones (an
-// iteration from a single-precision seed measured slower, and must
-// special-case zero strain).
-__device__ __forceinline__ double rcp_seed(double b)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-    return r;
-}
+// Reciprocals, square roots and maxima of the storage type: FP64 takes the short
+// sequences of les_fp64.cuh (the FP64 pipe is the bottleneck on this GPU); FP32
+// exists for the debug fields only.  Arguments are positive normal numbers
+// (densities, temperatures, sensor denominators), of roots and maxima
+// non-negative ones.
 template <typename real> __device__ __forceinline__ real rcp_(real b) { return real(1) / b; }
-template <> __device__ __forceinline__ double rcp_<double>(double b)
-{
-    double r = rcp_seed(b);
-    double e = fma(-b, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-b, r, 1.0);
-    return fma(r, e, r);
-}
+template <> __device__ __forceinline__ double rcp_<double>(double b) { return rcp64(b); }
 template <typename real> __device__ __forceinline__ real rcp1_(real b) { return real(1) / b; }
-template <> __device__ __forceinline__ double rcp1_<double>(double b)
-{
-    const double r = rcp_seed(b);
-    return fma(r, fma(-b, r, 1.0), r);
-}
+template <> __device__ __forceinline__ double rcp1_<double>(double b) { return rcp64_1(b); }
+template <typename real> __device__ __forceinline__ real sqrt_(real x) { return sqrt(x); }
+template <> __device__ __forceinline__ double sqrt_<double>(double x) { return sqrt64(x); }
+template <typename real> __device__ __forceinline__ real half_sqrt_(real x) { return real(0.5) * sqrt(x); }
+template <> __device__ __forceinline__ double half_sqrt_<double>(double x) { return half_sqrt64(x); }
+template <typename real> __device__ __forceinline__ real max_(real a, real b) { return fmax(a, b); }
+template <> __device__ __forceinline__ double max_<double>(double a, double b) { return max_nn(a, b); }
+template <typename real> __device__ __forceinline__ real pos_(real x) { return fmax(x, real(0)); }
+template <> __device__ __forceinline__ double pos_<double>(double x) { return clamp0(x); }
 
 // ---------------------------------------------------------------------------
 // k_point
@@ -96,7 +85,7 @@ __global__ void __launch_bounds__(BLOCK) k_point(const JetDev<real> *__restrict_
         const real gm1 = f64 ? (real)J.gm1 : gam - real(1);
         const real p = gm1 * (e - real(0.5) * (ru * u + rv * v + rw * w));
         const real T = gam * p * rrho;
-        const real sT = sqrt(T); // speed of sound: c^2 = gamma p / rho = T in jet units
+        const real sT = sqrt_<real>(T); // speed of sound: c^2 = gamma p / rho = T in jet units
         const real S = (real)J.suth_S;
         const real mu = T * sT * (f64 ? (real)J.suth1 : real(1) + S) * rcp1_<real>(T + S);
         const real rH = e + p;
@@ -119,7 +108,7 @@ __global__ void __launch_bounds__(BLOCK) k_point(const JetDev<real> *__restrict_
             F[4 * fs] = rH * hJU;
         }
         // lambda_a + (lambda_a lambda_b)^1/2 + (lambda_a lambda_d)^1/2 = s_a (s_a + s_b + s_d)
-        const real sq0 = sqrt(lam[0]), sq1 = sqrt(lam[1]), sq2 = sqrt(lam[2]);
+        const real sq0 = sqrt_<real>(lam[0]), sq1 = sqrt_<real>(lam[1]), sq2 = sqrt_<real>(lam[2]);
         const real ssum = sq0 + sq1 + sq2;
         P[P_RHO * fs + lp] = rho;
         P[P_U * fs + lp] = u;
@@ -156,36 +145,41 @@ __global__ void __launch_bounds__(BLOCK) k_grads(const JetDev<real> *__restrict_
         const real *__restrict__ P = J.prim;
         const real *__restrict__ M = J.met;
         real *__restrict__ G = J.grad;
-        real d[4][3]; // d phi / d xi^a, phi = u, v, w, T
+        real d[4][3]; // 2 d phi / d xi^a, phi = u, v, w, T
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const Stencil s = deriv_stencil(q[a], J.n[a], J.per[a]);
-            long long o[3];
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                int r[3] = {q[0], q[1], q[2]};
-                r[a] = J.per[a] ? wrapi(r[a] + s.off[t], J.n[a]) : r[a] + s.off[t];
-                o[t] = lidx(J, r[0], r[1], r[2]);
-            }
+            // central: the two neighbours; at an end of a non-periodic axis the
+            // points one and two inside (one-sided three-point)
+            const int n = J.n[a], per = J.per[a];
+            const bool end = !per && (q[a] == 0 || q[a] == n - 1);
+            const int t = q[a] == 0 ? 1 : -1;
+            int r1[3] = {q[0], q[1], q[2]}, r2[3] = {q[0], q[1], q[2]};
+            r1[a] = end ? q[a] + t : (per ? wrapi(q[a] - 1, n) : q[a] - 1);
+            r2[a] = end ? q[a] + 2 * t : (per ? wrapi(q[a] + 1, n) : q[a] + 1);
+            const long long o1 = lidx(J, r1[0], r1[1], r1[2]), o2 = lidx(J, r2[0], r2[1], r2[2]);
 #pragma unroll
             for (int f = 0; f < 4; ++f) {
                 const real *F = P + (f < 3 ? P_U + f : P_T) * fs;
-                real acc = (real)s.wgt[0] * F[o[0]] + (real)s.wgt[1] * F[o[1]];
-                if (s.n == 3) acc += (real)s.wgt[2] * F[o[2]];
-                d[f][a] = acc;
+                d[f][a] = F[o2] - F[o1];
             }
-            // pressure sensor along a; an end point of a non-periodic axis
-            // takes the sensor of its interior neighbour
-            int c = q[a];
-            if (!J.per[a]) c = c < 1 ? 1 : (c > J.n[a] - 2 ? J.n[a] - 2 : c);
-            int rm[3] = {q[0], q[1], q[2]}, r0[3] = {q[0], q[1], q[2]}, rp[3] = {q[0], q[1], q[2]};
-            r0[a] = c;
-            rm[a] = J.per[a] ? wrapi(c - 1, J.n[a]) : c - 1;
-            rp[a] = J.per[a] ? wrapi(c + 1, J.n[a]) : c + 1;
-            const real pm = P[P_P * fs + lidx(J, rm[0], rm[1], rm[2])];
-            const real p0 = P[P_P * fs + lidx(J, r0[0], r0[1], r0[2])];
-            const real pp = P[P_P * fs + lidx(J, rp[0], rp[1], rp[2])];
-            const real ps = pp + pm;
+            // a vote, so that the one-sided form stays a branch instead of
+            // predicated instructions at every point
+            if (__ballot_sync(__activemask(), end)) {
+                if (end) {
+                    const real td = t > 0 ? real(1) : real(-1);
+#pragma unroll
+                    for (int f = 0; f < 4; ++f) {
+                        const real *F = P + (f < 3 ? P_U + f : P_T) * fs;
+                        d[f][a] = td * fma(real(-3), F[lp], fma(real(3), F[o1], -d[f][a])); // t (4 f1 - 3 f0 - f2)
+                    }
+                }
+            }
+            // pressure sensor along a; an end point takes the sensor of its
+            // interior neighbour (the same three points)
+            const real *F = P + P_P * fs;
+            const real pl = F[lp], p1 = F[o1], p2 = F[o2];
+            const real p0 = end ? p1 : pl;
+            const real ps = p2 + (end ? pl : p1);
             G[(G_NU + a) * fs + lp] = fabs(fma(real(-2), p0, ps)) * rcp1_<real>(fma(real(2), p0, ps));
         }
 #pragma unroll
@@ -196,8 +190,8 @@ __global__ void __launch_bounds__(BLOCK) k_grads(const JetDev<real> *__restrict_
 #pragma unroll
         for (int t = 0; t < 9; ++t) m[t] = M[t * fs + lp];
         const real rj = M[MET_J * fs + lp];
-        // d u_i / d x_c = J g_ic with g_ic = sum_b m_bc d u_i / d xi^b (chain
-        // rule through the metric cofactors); 2 S_ij S_ij = J^2 (2 sum_i g_ii^2
+        // d u_i / d x_c = J g_ic / 2 with g_ic = sum_b m_bc d_ib (chain rule through
+        // the metric cofactors); 2 S_ij S_ij = (J/2)^2 (2 sum_i g_ii^2
         // + sum_{i<c} (g_ic + g_ci)^2)
         real g[3][3];
 #pragma unroll
@@ -215,7 +209,7 @@ __global__ void __launch_bounds__(BLOCK) k_grads(const JetDev<real> *__restrict_
             }
         }
         // Smagorinsky: mu_sgs = rho (Cs Delta)^2 (2 S_ij S_ij)^1/2
-        const real mus = P[P_RHO * fs + lp] * M[MET_CSD2 * fs + lp] * rj * sqrt(real(2) * sd + so);
+        const real mus = P[P_RHO * fs + lp] * M[MET_CSD2 * fs + lp] * rj * half_sqrt_<real>(real(2) * sd + so);
         const real mu = P[P_MU * fs + lp];
         G[G_MUSGS * fs + lp] = mus;
         G[G_MUEFF * fs + lp] = mu * (real)J.inv_Re + mus;
@@ -256,8 +250,8 @@ __device__ __forceinline__ void iface_flux(const JetDev<real> &J, const int qL[3
     }
     // Turkel-Vatsa: eps2 = k2 max(nu_L, nu_R), eps4 = max(0, k4 - eps2),
     // scaled by the interface lambda-bar and J^-1
-    const real eps2 = (real)J.k2 * fmax(G[(G_NU + a) * fs + L], G[(G_NU + a) * fs + R]);
-    const real eps4 = fmax(real(0), (real)J.k4 - eps2);
+    const real eps2 = (real)J.k2 * max_<real>(G[(G_NU + a) * fs + L], G[(G_NU + a) * fs + R]);
+    const real eps4 = pos_<real>((real)J.k4 - eps2);
     const real jbh = M[(MET_JB + a) * fs + L]; // half the interface J^-1
     const real sc = jbh * (P[(P_LXI + a) * fs + L] + P[(P_LXI + a) * fs + R]);
     const real se4 = sc * eps4;
@@ -280,9 +274,10 @@ __device__ __forceinline__ void iface_flux(const JetDev<real> &J, const int qL[3
     }
     // compact viscous + SGS flux: normal derivative from the two points,
     // tangential derivatives averaged, coefficients/metrics/velocity averaged.
-    // A = interface tables (cofactor average / interface J^-1, 1/2 folded into
+    // A = interface tables (cofactor average / interface J^-1, 1/4 folded into
     // the tangential rows), so grad phi = sum_b A_b D_b with D_a = phi_R - phi_L
-    // and D_b = the sum of the two points' central differences (b != a); the
+    // and D_b = the sum of the two points' stored doubled differences (b != a; the
+    // tables carry the 1/4); the
     // averaged cofactor row a is A_a times the interface J^-1, folded into the
     // transport coefficients.
     const real *__restrict__ A = M + (MET_A0 + 9 * a) * fs + L;
