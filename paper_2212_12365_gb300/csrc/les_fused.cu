@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
                 // the row norms |grad xi^a| / J; on the degenerate axis of a polar
                 // mesh (J^-1 = 0) J = 1 and the filter width is zero
                 const float2 jv = hi2(u[4]);
-                rj = make_float2(jv.x > 0.0f ? __fdividef(1.0f, jv.x) : 1.0f, jv.y > 0.0f ? __fdividef(1.0f, jv.y) : 1.0f);
+                rj = f2(jv.x > 0.0f ? rcpa(jv.x) : 1.0f, jv.y > 0.0f ? rcpa(jv.y) : 1.0f);
                 csdJ = make_float2(jv.x > 0.0f ? FP.cs2 * rcbrtf(jv.x) : 0.0f, jv.y > 0.0f ? FP.cs2 * rcbrtf(jv.y) : 0.0f);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
             // |S| = (2 S_ij S_ij)^1/2 = J sqrt(sd/2 + so/4) in terms of g'
             const float2 mus = mul2(mul2(rho, csdJ), sqrt2(fma2(so, bc(0.25f), mul2(sd, bc(0.5f)))));
             // Sutherland mu(T), speed of sound c = T^1/2
-            const float2 sT = sqrt2(T0);
+            const float2 sT = sqrtp2(T0);
             const float2 mu = mul2(mul2(T0, sT), mul2(bc(FP.suth1), rcp2(add2(T0, bc(FP.suthS)))));
             const float2 mue = fma2(mu, bc(FP.inv_Re), mus);
             const float2 kap = fma2(mu, bc(FP.kap_mol), mul2(mus, bc(FP.kap_sgs)));

@@ -38,14 +38,29 @@ __device__ __forceinline__ float4 cat4(float2 a, float2 b) { return make_float4(
 // thread's two rows
 __device__ __forceinline__ float2 odd2(float2 a, float2 b) { return make_float2(a.y, b.x); }
 __device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-// hardware approximate reciprocal (positive, normal arguments)
-__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y)); }
-// square root of x >= 0 through the hardware reciprocal square root
-// (max. 2 ulp): x * rsqrt(x), 0 -> 0 (a spectral radius vanishes on the axis
-// of a polar mesh)
+// Hardware reciprocal and reciprocal square root (1-2 ulp; arguments normal
+// numbers): the plain instructions, without the denormal handling that the
+// library wrappers put around them (about three instructions each; 17 pairs per
+// thread and plane in the general kernel)
+__device__ __forceinline__ float rcpa(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqa(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float2 rcp2(float2 a) { return f2(rcpa(a.x), rcpa(a.y)); }
+// x^1/2 = x rsqrt(x) for x > 0, and for x >= 0 (0 -> 0: no strain; a spectral
+// radius vanishes on the axis of a polar mesh)
+__device__ __forceinline__ float2 sqrtp2(float2 x) { return mul2(x, f2(rsqa(x.x), rsqa(x.y))); }
 __device__ __forceinline__ float2 sqrt2(float2 x)
 {
-    return mul2(x, make_float2(rsqrtf(fmaxf(x.x, 1.17549435e-38f)), rsqrtf(fmaxf(x.y, 1.17549435e-38f))));
+    return mul2(x, f2(rsqa(fmaxf(x.x, 1.17549435e-38f)), rsqa(fmaxf(x.y, 1.17549435e-38f))));
 }
 
 // Asynchronous 16-byte global -> shared copy, not kept in L1 (completes

@@ -100,27 +100,6 @@ template <int TY> struct PSm {
     }
 };
 
-// Hardware approximations without the denormal handling of the library
-// wrappers (arguments are normal numbers): 1/x and x^1/2 = x rsqrt(x), 1-2 ulp
-__device__ __forceinline__ float rcpa(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float rsqa(float x)
-{
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float2 rcpa2(float2 x) { return f2(rcpa(x.x), rcpa(x.y)); }
-__device__ __forceinline__ float2 sqrta2(float2 x) { return mul2(x, f2(rsqa(x.x), rsqa(x.y))); } // x > 0
-__device__ __forceinline__ float2 sqrt0a2(float2 x)                                              // x >= 0
-{
-    return mul2(x, f2(rsqa(fmaxf(x.x, 1.17549435e-38f)), rsqa(fmaxf(x.y, 1.17549435e-38f))));
-}
-
 // One point pair: velocity, p - p_inf, density, rho H, T, and rho u.
 struct PP {
     float2 u[3], p, rho, rH, T, m[3];
@@ -290,7 +269,7 @@ __global__ void __launch_bounds__(FX *TY / 2, 1)
         const float hbx_ = __fmul_rn(0.5f, __fadd_rn(hx0.x, hx1.x)), rhbx_ = __fmul_rn(4.0f, rcpa(hbx_));
         const float2 hbx = bc(hbx_), rhbx = bc(rhbx_), c43x = bc(__fmul_rn(4.0f / 3.0f, rhbx_));
         const float2 hby = mul2(bc(0.5f), add2(f2(hyA0.x, hyB0.x), f2(hyA1.x, hyB1.x)));
-        const float2 rhby = mul2(bc(4.0f), rcpa2(hby)), c43y = mul2(bc(4.0f / 3.0f), rhby);
+        const float2 rhby = mul2(bc(4.0f), rcp2(hby)), c43y = mul2(bc(4.0f / 3.0f), rhby);
         // (Cs Delta)^2 / 4 less its k factor (the 1/4 of the coefficients)
         const float2 csxy = mul2(bc(__fmul_rn(__fmul_rn(0.25f, FP.cs2), hx0.z)), f2(hyA0.z, hyB0.z));
 
@@ -337,7 +316,7 @@ __global__ void __launch_bounds__(FX *TY / 2, 1)
         auto sensor = [&](float2 pm, float2 pc, float2 pp) { // of p - p_inf
             const float2 s = add2(pm, pp);
             const float2 num = fma2(pc, bc(-2.0f), s), den = fma2(pc, bc(2.0f), add2(s, bc(pinf4)));
-            const float2 r = rcpa2(den);
+            const float2 r = rcp2(den);
             return mul2(bc(FP.k2), f2(__fmul_rn(fabsf(num.x), r.x), __fmul_rn(fabsf(num.y), r.y)));
         };
         // one-sided at an end: cells c (own), c1, c2 one and two inside, t = +-1
@@ -400,7 +379,7 @@ __global__ void __launch_bounds__(FX *TY / 2, 1)
                     }
                     const float2 rho = f2(q[0][0], q[1][0]), e = f2(q[0][4], q[1][4]);
                     const float2 m[3] = {f2(q[0][1], q[1][1]), f2(q[0][2], q[1][2]), f2(q[0][3], q[1][3])};
-                    const float2 rr = rcpa2(rho);
+                    const float2 rr = rcp2(rho);
                     const float2 u = mul2(m[0], rr), v = mul2(m[1], rr), w = mul2(m[2], rr);
                     const float2 ke2 = fma2(m[2], w, fma2(m[1], v, mul2(m[0], u)));
                     // p rounded before p_inf is taken off, as in the general form: the
@@ -499,16 +478,16 @@ __global__ void __launch_bounds__(FX *TY / 2, 1)
                     const float2 sd = fma2(D[2][2], D[2][2], fma2(D[1][1], D[1][1], mul2(D[0][0], D[0][0])));
                     const float2 so = fma2(a12, a12, fma2(a02, a02, mul2(a01, a01)));
                     // mu_sgs / 4 = rho (Cs Delta)^2 / 4 (2 S_ij S_ij)^1/2
-                    const float2 mus = mul2(mul2(O.rho, mul2(csxy, bc(hz.z))), sqrt0a2(fma2(so, bc(0.25f), mul2(sd, bc(0.5f)))));
-                    const float2 sT = sqrta2(O.T); // speed of sound
-                    const float2 mu4 = mul2(mul2(O.T, sT), mul2(bc(__fmul_rn(0.25f, FP.suth1)), rcpa2(add2(O.T, bc(FP.suthS)))));
+                    const float2 mus = mul2(mul2(O.rho, mul2(csxy, bc(hz.z))), sqrt2(fma2(so, bc(0.25f), mul2(sd, bc(0.5f)))));
+                    const float2 sT = sqrtp2(O.T); // speed of sound
+                    const float2 mu4 = mul2(mul2(O.T, sT), mul2(bc(__fmul_rn(0.25f, FP.suth1)), rcp2(add2(O.T, bc(FP.suthS)))));
                     X.mue = fma2(mu4, bc(FP.inv_Re), mus);
                     X.kap = fma2(mu4, bc(FP.kap_mol), mul2(mus, bc(FP.kap_sgs)));
                     // lambda_a = (|u_a| + c) / |h_a|; lambda-bar_a = s_a (s_a + s_b + s_d)
                     float2 sq[3];
 #pragma unroll
                     for (int a = 0; a < 3; ++a)
-                        sq[a] = sqrta2(f2(__fmul_rn(__fadd_rn(fabsf(O.u[a].x), sT.x), fabsf(rh[a].x)),
+                        sq[a] = sqrtp2(f2(__fmul_rn(__fadd_rn(fabsf(O.u[a].x), sT.x), fabsf(rh[a].x)),
                                          __fmul_rn(__fadd_rn(fabsf(O.u[a].y), sT.y), fabsf(rh[a].y))));
                     const float2 ss = add2(add2(sq[0], sq[1]), sq[2]);
                     Y.mue = Z.mue = X.mue;
