@@ -252,18 +252,18 @@ __device__ __forceinline__ void inflow_state(const JetDev<real> &J, T ut, T g, T
     }
 }
 
-// Boundary state Qf at face point F (indices q) of `axis` and `side` from the
+// Boundary state Qf at face point q of `axis` and `side`, metric row n, from the
 // unscaled state Qe of its inner neighbour.
 template <typename real, typename T>
-__device__ __forceinline__ void face_state(const JetDev<real> &J, int axis, int side, long long F, const int q[3],
+__device__ __forceinline__ void face_state(const JetDev<real> &J, int axis, int side, T n[3], const int q[3],
                                            long long level, const T Qe[5], T Qf[5])
 {
     const int type = J.bc[2 * axis + side];
-    // unit outward normal from the face point's metric row
-    T n[3], nn = T(0);
+    // unit outward normal from the face point's metric row n
+    T nn = T(0);
     const T sg = side ? T(1) : T(-1);
     for (int c = 0; c < 3; ++c) {
-        n[c] = sg * J.met[(3 * axis + c) * J.fs + F];
+        n[c] *= sg;
         nn = fma(n[c], n[c], nn);
     }
     const bool inflow = type == LES_BC_INFLOW_JET;
@@ -309,13 +309,14 @@ __device__ __forceinline__ void face_state(const JetDev<real> &J, int axis, int 
 // stage whose 256-thread blocks left a small face on a dozen SMs, bound by the
 // FP64 issue of those SMs; blocks of 64 spread every face over the chip.
 // Measured per stage: FP64 48x32x32 95 -> 21 us (a traced launch costs 6 of
-// them), 384x256x144 242 -> 117 us; FP32 192x128x72 37 -> 19 us.
+// them), 384x256x144 242 -> 131 us; FP32 192x128x72 37 -> 12 us.
 constexpr int BC_BLOCK = 64;
+// (32-bit face indices: a face has fewer points than a jet, and those fit.)
 // Thread t of a jet's boundary pass: false if it has no point; else F, the
 // padded index of its face point, and Q, the stored boundary state there, from
 // the interior points of buffer Qs.
 template <typename real>
-__device__ __forceinline__ bool bc_point(const JetDev<real> &J, long long t, long long level, const real *Qs,
+__device__ __forceinline__ bool bc_point(const JetDev<real> &J, int t, long long level, const real *Qs,
                                          long long &F, real Q[5])
 {
     using T = real;
@@ -327,11 +328,11 @@ __device__ __forceinline__ bool bc_point(const JetDev<real> &J, long long t, lon
         const int a = s == 0 ? 0 : 3 - s;
         if (J.per[a] || axis >= 0) continue;
         const int b = a == 0 ? 1 : 0, d = a == 2 ? 1 : 2;
-        const long long nface = (long long)J.n[b] * J.n[d];
+        const int nface = J.n[b] * J.n[d];
         if (t < 2 * nface) {
             axis = a;
             const int side = t >= nface;
-            const int r = (int)(t - side * nface);
+            const int r = t - side * nface;
             const int id = r / J.n[b];
             q[a] = side ? J.n[a] - 1 : 0;
             q[b] = r - id * J.n[b];
@@ -353,6 +354,25 @@ __device__ __forceinline__ bool bc_point(const JetDev<real> &J, long long t, lon
     }
     if (!on[axis] || (axis != 0 && on[0]) || (axis == 1 && on[2])) return false;
     const long long fs = J.fs;
+    // In FP32 everything the chain reads is fetched before it, the metric rows of
+    // the faces the point lies on too: one memory latency instead of one per face
+    // (48x32x32 9.5 -> 8.3 us, 192x128x72 13.8 -> 11.9 us).  In FP64 the rows are
+    // read face by face: nine more doubles held cost warps
+    // (384x256x144 131 -> 137 us).
+    constexpr bool AHEAD = sizeof(real) == sizeof(float);
+    T nr[3][3];
+    if (AHEAD) {
+        int at[3] = {cur[0], cur[1], cur[2]};
+#pragma unroll
+        for (int s = 1; s < 4; ++s) {
+            const int a = s == 3 ? 0 : s;
+            if (!on[a]) continue;
+            at[a] = q[a];
+            const long long o = lidx(J, at[0], at[1], at[2]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) nr[a][c] = J.met[(3 * a + c) * fs + o];
+        }
+    }
     {
         const long long E = lidx(J, cur[0], cur[1], cur[2]);
         const T rs = sizeof(real) == sizeof(float) ? T(1) : (T)J.met[MET_J * fs + E];
@@ -361,10 +381,19 @@ __device__ __forceinline__ bool bc_point(const JetDev<real> &J, long long t, lon
 #pragma unroll 1
     for (int s = 1; s < 4; ++s) { // y, z, x
         const int a = s == 3 ? 0 : s;
-        if (!on[a]) continue;
-        cur[a] = q[a];
-        T Qf[5];
-        face_state<real, T>(J, a, q[a] != 0, lidx(J, cur[0], cur[1], cur[2]), q, level, Q, Qf);
+        if (!(s == 1 ? on[1] : (s == 2 ? on[2] : on[0]))) continue;
+        const int qa = s == 1 ? q[1] : (s == 2 ? q[2] : q[0]);
+        T n[3], Qf[5];
+        if (AHEAD) {
+            for (int c = 0; c < 3; ++c) n[c] = s == 1 ? nr[1][c] : (s == 2 ? nr[2][c] : nr[0][c]);
+        } else {
+            if (s == 1) cur[1] = qa;
+            else if (s == 2) cur[2] = qa;
+            else cur[0] = qa;
+            const long long o = lidx(J, cur[0], cur[1], cur[2]);
+            for (int c = 0; c < 3; ++c) n[c] = J.met[(3 * a + c) * fs + o];
+        }
+        face_state<real, T>(J, a, qa != 0, n, q, level, Q, Qf);
         for (int f = 0; f < 5; ++f) Q[f] = Qf[f];
     }
     F = lidx(J, q[0], q[1], q[2]);

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(BC_BLOCK) k_bc(const JetDev<real> *__restrict_
     const int b0 = ONE ? 0 : bm.start[jet];
     long long F;
     real Q[5];
-    if (!bc_point(J, (long long)(blockIdx.x - b0) * BC_BLOCK + threadIdx.x, *level_p, J.q[dst], F, Q)) return;
+    if (!bc_point(J, (int)(blockIdx.x - b0) * BC_BLOCK + (int)threadIdx.x, *level_p, J.q[dst], F, Q)) return;
     for (int f = 0; f < 5; ++f) J.q[dst][f * J.fs + F] = Q[f];
 }
 
