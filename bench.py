@@ -42,11 +42,33 @@ from paper_2212_12365_gb300 import inputs as I  # noqa: E402
 # in the update and those three 1/2 factors per interface: 711.
 FLOPS_PER_PT_STAGE = {"point": 94, "grads": 112, "iface": 465, "update": 35}
 FLOPS_PER_PT_STAGE_FUSED = 711
+# The same count for the form that Cartesian-product grids take (diagonal
+# metrics, fluxes divided by the face area): point pass 52 (scaling 5,
+# primitives, Sutherland and rho H 18, six momentum and three energy fluxes 12,
+# spectral radii and lambda-bar 17), gradients and closures 65 (differences 9,
+# sensors 21, scaling and strain 22, closures 13), three interface fluxes
+# 3 x 77 = 231 (dissipation 42, viscous rows 19, energy 16), update 50 (three
+# face factors 5, fifteen differences and FMAs 45): 398.  FP32: no scaling, and
+# three factors instead of five operations for the faces: 391.
+FLOPS_PER_PT_STAGE_PRODUCT = {"point": 52, "grads": 65, "iface": 231, "update": 50}
+FLOPS_PER_PT_STAGE_FUSED_PRODUCT = 391
 # Algorithmic HBM bytes per point and stage: stages 2-5 read Q(l-1), Q(0) and 10
 # metric values and write Q(l); stage 1 reads Q(0) once: 24 values on average.
-ALGO_BYTES_PER_PT_STAGE = {"fp64": 24 * 8, "fp32": 24 * 4,
-                           # separable metrics (product grids): no 3-D metric fields, 14 values
-                           "fp32-sep": 14 * 4}
+# On a product grid the spacings are 1-D tables: 14 values.
+VALUES_PER_PT_STAGE, VALUES_PER_PT_STAGE_PRODUCT = 24, 14
+
+
+def algo_bytes_per_pt_stage(prec: str, describe: str) -> int:
+    """Algorithmic HBM bytes per point and stage of the form that les_describe names."""
+    n = VALUES_PER_PT_STAGE_PRODUCT if is_product(describe) else VALUES_PER_PT_STAGE
+    return n * (8 if prec == "fp64" else 4)
+
+
+def is_product(describe: str) -> bool:
+    """Whether the handle's jets (all of them) run the product-grid stage."""
+    return "(product)" in describe or "fused product" in describe and "fused general" not in describe
+
+
 # DRAM bytes per point of one launch of the dominant kernel in the launch
 # configuration of the run, from the ncu captures summarised in profiles/:
 # keyed by workload, precision, kernel and (fused stage) the decomposition in
@@ -54,15 +76,14 @@ ALGO_BYTES_PER_PT_STAGE = {"fp64": 24 * 8, "fp32": 24 * 4,
 # at capture time; when the file has changed since, the figure no longer
 # describes the kernel that runs and the lookup gives None.
 _PAPER_JET = "jet-384x256x144"
-KERNEL_SOURCE = {"k_iface": "les_stage.cu", "k_fused": "les_fused.cu"}
+KERNEL_SOURCE = {"k_iface": "les_stage.cu", "k_fused": "les_fused.cu",
+                 "k_iface_prod": "les_stage_prod.cu", "k_fused_prod": "les_fused_prod.cu"}
 TRAFFIC_BYTES_PER_POINT = {  # (workload, precision, kernel, decomposition) -> (bytes per point, source sha16)
-    # profiles/stage_kernels_fp64_jet-384x256x144.md: 13415.1 + 1682.3 MB per launch
-    (_PAPER_JET, "fp64", "k_iface", None): (1066.51, "e93049f182835582"),
-    # profiles/fused_stage_fp32_jet-384x256x144.md and ..._separable_...
-    (_PAPER_JET, "fp32", "k_fused", "ty=16 kc=balanced"): (128.55, "2231f6aa9a29f415"),
-    (_PAPER_JET, "fp32", "k_fused", "ty=16 kc=lockstep"): (106.47, "2231f6aa9a29f415"),
-    (_PAPER_JET, "fp32-sep", "k_fused", "ty=16 kc=balanced"): (77.23, "2231f6aa9a29f415"),
-    (_PAPER_JET, "fp32-sep", "k_fused", "ty=16 kc=lockstep"): (55.67, "2231f6aa9a29f415"),
+    # profiles/stage_kernels_fp64_product_jet-384x256x144.md: 4337.4 + 1647.3 MB per launch
+    (_PAPER_JET, "fp64", "k_iface_prod", None): (422.77, "06f31f685abc74c4"),
+    # profiles/fused_stage_fp32_product_jet-384x256x144.md: mean of the five stages
+    (_PAPER_JET, "fp32", "k_fused_prod", "ty=24 kc=balanced"): (62.63, "dfa4e15cca376cd6"),
+    (_PAPER_JET, "fp32-sep", "k_fused_prod", "ty=24 kc=balanced"): (62.63, "dfa4e15cca376cd6"),
 }
 
 
@@ -99,16 +120,9 @@ def traffic_bytes_per_point(workload: str, prec: str, kname: str, describe: str,
 # captures (sm__inst_executed_pipe_*, % of peak sustained while active), with
 # the source hash of the captured kernel as above
 PIPE_UTIL_NCU = {  # (precision, kernel) -> (metrics dict, source sha16)
-    # profiles/stage_kernels_fp64_jet-384x256x144.md (192x128x72 capture)
-    ("fp64", "k_iface"): ({"fp64_pipe_pct": 88.82, "executed_fp64_flop_per_point": 459.8,
-                          "dadd_dmul_dfma_per_point": [118.9, 67.4, 136.8]}, "e93049f182835582"),
-    # profiles/fused_stage_fp32_jet-384x256x144.md (192x128x72 capture, 32x16 tiles)
-    ("fp32", "k_fused"): ({"fma_pipe_pct": 33.8, "fmaheavy_pct": 33.0, "fmalite_pct": 34.0, "issue_active_pct": 37.8,
-                          "executed_fp32_flop_per_point": 1320.6, "thread_instructions_per_point": 1087.1},
-                         "2231f6aa9a29f415"),
-    ("fp32-sep", "k_fused"): ({"fma_pipe_pct": 32.6, "fmaheavy_pct": 34.7, "fmalite_pct": 30.1,
-                              "issue_active_pct": 40.5, "executed_fp32_flop_per_point": 819.8,
-                              "thread_instructions_per_point": 858.0}, "2231f6aa9a29f415"),
+    # profiles/stage_kernels_fp64_product_jet-384x256x144.md (192x128x72 capture)
+    ("fp64", "k_iface_prod"): ({"fp64_pipe_pct": 87.9, "fp64_instructions_per_point": 162.0,
+                                "issue_active_pct": 15.0}, "06f31f685abc74c4"),
 }
 # Nominal multiply-add throughput of GB300 (unit counts x the maximum clock),
 # reported beside the measured figures: 2 DFMA and 128 FFMA per clock and SM.
@@ -363,7 +377,8 @@ def _time_steps(solver, steps, torch):
 def batched_form(args, les, torch, fp64_value):
     """The batched form (64 jets of uneven grids, Mach, temperature ratio,
     Reynolds number and seed, one persistent launch per stage, the step a
-    CUDA graph), FP32 and FP32 with separable metrics: device rate after the
+    CUDA graph), LES_FP32 and LES_FP32_SEPARABLE (the same kernel on these
+    grids): device rate after the
     warm-up, the HBM fraction of the algorithmic bytes, and a bit-for-bit
     check of three jets against single-jet handles after the same steps."""
     specs, fps = _batch64()
@@ -389,7 +404,7 @@ def batched_form(args, les, torch, fp64_value):
         ms = _time_steps(b, args.steps, torch)
         v = N * 5 * args.steps / (ms / 1e3)
         out[name] = {"value": v, "ms_per_step": ms / args.steps, "speedup_vs_fp64_single_jet": v / fp64_value,
-                     "hbm_frac_algorithmic": v * ALGO_BYTES_PER_PT_STAGE[name] / 1e9 / hbm,
+                     "hbm_frac_algorithmic": v * algo_bytes_per_pt_stage(name, les.les_describe(b.h)) / 1e9 / hbm,
                      "bit_identical_to_single_jets": {"jets": list(check_jets), "after_steps": nchk,
                                                       "equal": same},
                      "stage": les.les_describe(b.h)}
@@ -415,7 +430,7 @@ def large_probe_form(args, les, torch):
     hbm, _ = hbm_peak_gbs()
     out = {"workload": "jet-768x384x192", "precision": "fp32", "points": spec.N, "value": v,
            "ms_per_step": ms / args.steps,
-           "hbm_frac_algorithmic": v * ALGO_BYTES_PER_PT_STAGE["fp32"] / 1e9 / hbm,
+           "hbm_frac_algorithmic": v * algo_bytes_per_pt_stage("fp32", les.les_describe(s.h)) / 1e9 / hbm,
            "probe": {"points": int(xyz.shape[1]), "every": 5, "frames": int(frames),
                      "finite": bool(torch.isfinite(ring).all().item())},
            "stage": les.les_describe(s.h)}
@@ -424,9 +439,10 @@ def large_probe_form(args, les, torch):
 
 
 # FP32 operations per (panel, observer, time) evaluation of the FW-H observer
-# pass: emission-frame position 2, seven retarded interpolations 21, the two
-# radial projections 10, the integrand 5, the compensated sum 4.
-FWH_FLOP_PER_EVAL = 42
+# pass: the integrand of a frame 13 (formed once per panel, microphone and
+# frame; one frame per observer time here), emission-frame position 4, one
+# retarded interpolation 3, the compensated sum 4.
+FWH_FLOP_PER_EVAL = 24
 
 
 def fwh_form(les, torch, alu):
@@ -536,9 +552,10 @@ def precision_form(args, spec, fp, les, torch, fp64_value):
         f["speedup_vs_fp64"] = f["value"] / fp64_value
         f["rel_l2_vs_fp64_per_field"] = [float(e) for e in err]
         f["after_steps"] = steps
-        f["hbm_frac_algorithmic"] = f["value"] * ALGO_BYTES_PER_PT_STAGE[names[prec]] / 1e9 / hbm_peak_gbs()[0]
+        f["hbm_frac_algorithmic"] = (f["value"] * algo_bytes_per_pt_stage(f["precision"], f["stage"]) / 1e9
+                                     / hbm_peak_gbs()[0])
     out = forms[les.LES_FP32]
-    # the separable-metric stage (Cartesian-product grids only), reported apart
+    # LES_FP32_SEPARABLE (Cartesian-product grids only), reported apart
     out["separable"] = forms[les.LES_FP32_SEPARABLE]
     return out
 
@@ -608,22 +625,26 @@ def run_ours(args):
     prof = les.les_profile_step(solver.h, max(1, min(args.steps, 3)))
     tot = sum(v[0] for v in prof.values())
     alu = alu_peaks(les)
+    describe = les.les_describe(solver.h)
+    prod = is_product(describe)
     if prec == "fp64":
         dom = max(FLOPS_PER_PT_STAGE, key=lambda k: prof[k][0])
-        kname, flops_pt = f"k_{dom}", FLOPS_PER_PT_STAGE[dom]
+        kname = f"k_{dom}_prod" if prod else f"k_{dom}"
+        flops_pt = (FLOPS_PER_PT_STAGE_PRODUCT if prod else FLOPS_PER_PT_STAGE)[dom]
         peak, peak_nominal = alu["fp64_fma"], FP64_NOMINAL_TFLOPS
         peak_source = "measured: DFMA loop of les_measure_peak on this GPU (CUDA events)"
     else:
         dom = "iface"  # the fused single-pass stage kernel is traced under this kind
-        kname, flops_pt = "k_fused", FLOPS_PER_PT_STAGE_FUSED
+        kname = "k_fused_prod" if prod else "k_fused"
+        flops_pt = FLOPS_PER_PT_STAGE_FUSED_PRODUCT if prod else FLOPS_PER_PT_STAGE_FUSED
         peak, peak_nominal = alu["fp32_fma"], FP32_NOMINAL_TFLOPS
         peak_source = "measured: FFMA loop of les_measure_peak on this GPU (CUDA events)"
     t_launch = prof[dom][0] / max(prof[dom][1], 1) / 1e3  # s per launch
     achieved = flops_pt * N / t_launch / 1e12
     hbm_peak, hbm_source = hbm_peak_gbs()
-    traffic_pt = traffic_bytes_per_point(args.workload, prec, kname, les.les_describe(solver.h))
+    traffic_pt = traffic_bytes_per_point(args.workload, prec, kname, describe)
     pipe = PIPE_UTIL_NCU.get((prec, kname))
-    bytes_pt_stage = ALGO_BYTES_PER_PT_STAGE[prec]
+    bytes_pt_stage = algo_bytes_per_pt_stage(prec, describe)
     roofline = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic_pt * N if traffic_pt else None,
                 "pipe_util_ncu": pipe[0] if pipe and pipe[1] == source_sha16(kname) else None,
@@ -633,7 +654,7 @@ def run_ours(args):
                 "flops_per_point_stage": flops_pt,
                 "share": prof[dom][0] / tot if tot else None,
                 "per_kernel_ms_per_launch": {k: v[0] / max(v[1], 1) for k, v in prof.items() if v[1]},
-                "stage": les.les_describe(solver.h),
+                "stage": describe,
                 "source_sha16": source_sha16(kname),
                 # the metric's "% HBM roofline": algorithmic bytes of a stage at the achieved rate
                 "hbm_view": {"algorithmic_bytes_per_point_stage": bytes_pt_stage,
@@ -759,7 +780,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default="jet-384x256x144", choices=sorted(WORKLOADS))
     ap.add_argument("--precision", default=None, choices=["fp64", "fp32", "fp32-sep"],
-                    help="fp32-sep: FP32 with the separable-metric stage (product grids)")
+                    help="fp32-sep: LES_FP32_SEPARABLE (product grids only)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-fp32", action="store_true", help="skip the FP32 line of the FP64 default run")

@@ -71,12 +71,14 @@ extern "C" {
  * Jacobian are always computed in FP64; diagnostics sum in FP64. */
 #define LES_FP64 0
 #define LES_FP32 1
-/* FP32 with the separable-metric stage: only for a Cartesian-product grid
- * (x depends on i only, y on j only, z on k only; LES_ERR_ARG otherwise).
- * The cofactors are then diagonal products of the three 1-D spacings
- * dx/dxi, dy/deta, dz/dzeta (Sec. "Transformation of Coordinates"), which the
- * stage kernel reads from three 1-D tables instead of nine stored fields;
- * everything else behaves as LES_FP32 (state kinds, probe, diagnostics). */
+/* FP32 that insists on a Cartesian-product grid (x depends on i only, y on j
+ * only, z on k only; LES_ERR_ARG otherwise).  The cofactors are then diagonal
+ * products of the three 1-D spacings dx/dxi, dy/deta, dz/dzeta (Sec.
+ * "Transformation of Coordinates"), which the stage kernel reads from three
+ * 1-D tables instead of nine stored fields.  LES_FP64 and LES_FP32 handles
+ * take that form by themselves for every jet on such a grid with positive
+ * spacings and run the general metrics for the others; everything else
+ * behaves as LES_FP32 (state kinds, probe, diagnostics). */
 #define LES_FP32_SEPARABLE 2
 
 /* State kinds for les_set_state / les_get_state. */
@@ -239,7 +241,7 @@ int les_profile_step(les_handle *h, int nsteps, double *ms_out, int64_t *counts)
 
 /* Work decomposition of the fused FP32 stage (LES_FP32, LES_FP32_SEPARABLE
  * handles): ty = 8 or 16 grid rows per CTA tile (32 x ty/2 threads, two rows
- * each), kc >= 1
+ * each; the tuner also tries 24 for jets on product grids), kc >= 1
  * planes per k-chunk item, kc = 0 for the balanced form (every CTA of the
  * persistent grid takes one contiguous, equal share of all tile-planes), or
  * kc = -1 for the lockstep form (whole columns in waves of one tile per CTA,
@@ -363,8 +365,9 @@ int les_fwh(const void *ring, int precision, int capacity, int64_t frames_writte
             double t0, double dt_obs, int nt, double *p_out, void *stream, double *ms_out);
 
 /* Human-readable description of a handle: precision, jets, device bytes and
- * the stage kernel configuration chosen by the autotuner (FP32: fused tile
- * height and k-chunk; FP64: four-kernel stage).  Valid until the next call
+ * the form of the stage (product-grid or general metrics; "general, product"
+ * for a batch of both) with the configuration chosen by the autotuner (FP32:
+ * fused tile height and k-chunk; FP64: four-kernel stage).  Valid until the next call
  * on the handle. */
 const char *les_describe(les_handle *h);
 
