@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "les_fp64.cuh"
+#include "les_fwh_plan.h"
 #include "les_internal.cuh"
 #include "les_pair.cuh"
 
@@ -35,7 +36,6 @@ namespace les {
 
 namespace {
 
-constexpr int FWH_T = 256;   // observer times per CTA
 constexpr int FWH_SUB = 256; // panels per shared-memory sub-chunk
 
 // Ring frame m (0 = oldest used) of field f at panel j.
@@ -296,8 +296,6 @@ __global__ void __launch_bounds__(FWH_T) k_fwh_obs(const float4 *__restrict__ sr
 // shared-memory wavefront limit (66 %); now an evaluation reads 8 bytes and the
 // pass is bound by issue and barriers at 16 warps per SM (issue 48 %, shared
 // memory 54 %).  98,304 panels, 64 microphones, 512 times: 11.4 -> 4.7 ms.
-constexpr int FWH_MG = 16;  // microphones per group, at most
-constexpr int FWH_PB = 8;   // panels whose geometry is staged together
 __device__ __forceinline__ float2 fadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -308,17 +306,14 @@ __device__ __forceinline__ void fwh_cp16(void *dst, const void *src)
                  : "memory");
 }
 
-// Shared memory of the staged pass for windows of W entries (a multiple of 32).
+// Staged geometry of a panel.
 struct FwhGeo {
     float4 pair[FWH_MG / 2][3]; // microphones 2p, 2p+1: (glx, glx', gly, gly') (glz, glz', gw, gw') (q, q', -, -)
     float4 off[FWH_MG];         // fraction (twice), offset in the window (int bits), -
     unsigned mask[32];          // microphone pairs that read the window's entries 32 w .. 32 w + 31
     int base, pad[3];           // frame of the window's first entry
 };
-__host__ __device__ constexpr size_t fwh_win_smem(int W) // V twice, the records, the geometry
-{
-    return 4 * ((size_t)2 * FWH_MG * W) + 32 * (size_t)W + FWH_PB * sizeof(FwhGeo);
-}
+static_assert(sizeof(FwhGeo) == FWH_GEO_BYTES, "fwh_win_smem counts it");
 
 // FULL: every group has sixteen microphones.
 template <int NTH, bool FULL>
@@ -328,8 +323,9 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_fwh_obs_win(const float4 *__
                                                       int span, int add, double *__restrict__ part)
 {
     extern __shared__ __align__(16) float fwh_sm[];
-    float *V = fwh_sm;                             // [2][FWH_MG][W]
-    float4 *RA = (float4 *)(V + 2 * FWH_MG * W);   // [W] records of the next panel: (L, dQ/dtau)
+    const int rows = FULL ? FWH_MG : (MG + 1) / 2 * 2; // fwh_rows
+    float *V = fwh_sm;                             // [2][rows][W]
+    float4 *RA = (float4 *)(V + 2 * rows * W);     // [W] records of the next panel: (L, dQ/dtau)
     float4 *RB = RA + W;                           // [W]: dL/dtau
     FwhGeo *G = (FwhGeo *)(RB + W);                // [FWH_PB]
     const int tid = threadIdx.x;
@@ -358,7 +354,7 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_fwh_obs_win(const float4 *__
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    float *Vb = V, *Vn = V + FWH_MG * W;
+    float *Vb = V, *Vn = V + rows * W;
     for (int jb = j0; jb < j1; jb += FWH_PB) {
         const int np = min(FWH_PB, j1 - jb);
         __syncthreads(); // the previous panels' geometry is no longer read
@@ -508,10 +504,7 @@ extern "C" int les_fwh(const void *ring, int precision, int capacity, int64_t fr
     int dev = 0, nsm = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return LES_ERR_CUDA;
-    // microphone groups of equal size, at most 16
-    const int ngroups = (nobs + FWH_MG - 1) / FWH_MG, MG = (nobs + ngroups - 1) / ngroups;
-    // panels per batch: source records of at most 256 MB (and at least 1024 panels)
-    const int NB = (int)std::min<long long>(npts, std::max<long long>(1024, (256LL << 20) / (32LL * N) / 256 * 256));
+    const int MG = fwh_group(nobs);
     const size_t n_out = (size_t)nobs * nt;
     double *d_geo = nullptr;   // panel geometry, microphones, distance limits
     char *d_work = nullptr;    // batch records, partial sums, result
@@ -563,30 +556,11 @@ extern "C" int les_fwh(const void *ring, int precision, int capacity, int64_t fr
             return bad(msg);
         }
     }
-    // The staged observer pass: blocks of up to 512 observer times, in equal
-    // parts; per panel a window of W frames (the block's times plus the spread
-    // of the group's emission times).  Two CTAs of 256 threads fit an SM by
-    // their registers, so a CTA may use 110 KB of shared memory; when the times
-    // are so sparse that the window takes more, the direct pass.
-    const int tblocks = (nt + 511) / 512, T = (nt + tblocks - 1) / tblocks;
-    const double span_d = std::floor((T - 1) * dt_obs / dtau + 2.0) + 1.0;
-    const double W_d = span_d + std::ceil(lim[2 * nobs] / (c0 * dtau)) + 6.0;
-    const int W_r = W_d < 4096.0 ? ((int)W_d + 31) / 32 * 32 : 4096;
-    const bool staged = W_r <= 1024 && fwh_win_smem(W_r) <= 110 * 1024;
-    const int W = staged ? W_r : 0, span = staged ? (int)span_d : 0;
-    const int tb = staged ? tblocks : (nt + FWH_T - 1) / FWH_T;
-    // threads: half the block's times, so that few are idle in a short block
-    const int nth = T <= 128 ? 64 : (T <= 256 ? 128 : 256);
-    // panel chunks of a batch: the CTAs of one wave (staged: 512 threads or the
-    // shared memory of an SM; direct: four CTAs per SM)
-    const int cps = staged ? std::min(512 / nth, (int)(220 * 1024 / fwh_win_smem(W))) : 4;
-    int nchunk = staged ? cps * nsm / (tb * ngroups) : (cps * nsm + tb * nobs - 1) / (tb * nobs);
-    nchunk = std::max(1, std::min(nchunk, (NB + FWH_PB - 1) / FWH_PB));
-    const size_t b_src = (size_t)NB * N * 32, b_rec = staged ? (size_t)NB * nobs * 32 : 0,
-                 b_part = n_out * (nchunk + 1) * sizeof(double);
-    if (cudaMalloc(&d_work, b_src + b_rec + b_part) != cudaSuccess) return oom();
-    float4 *d_src = (float4 *)d_work, *d_rec = (float4 *)(d_work + b_src);
-    double *d_part = (double *)(d_work + b_src + b_rec), *d_out = d_part + n_out * nchunk;
+    const FwhPlan P = fwh_plan(npts, N, nobs, nt, dt_obs, dtau, c0, lim[2 * nobs], nsm);
+    const int NB = P.NB, nchunk = P.nchunk;
+    if (cudaMalloc(&d_work, P.scratch()) != cudaSuccess) return oom();
+    float4 *d_src = (float4 *)d_work, *d_rec = (float4 *)(d_work + P.b_src);
+    double *d_part = (double *)(d_work + P.b_src + P.b_rec), *d_out = d_part + n_out * nchunk;
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     int rc = LES_OK;
     if (ms_out) {
@@ -608,21 +582,20 @@ extern "C" int les_fwh(const void *ring, int precision, int capacity, int64_t fr
             k_fwh_src<float><<<gs, 128, 0, st>>>((const float *)ring, first, capacity, npts, j0, nb, N, d_nrm, p0, rdt2,
                                                  d_src);
         if (ms_out) cudaEventRecord(ev[1], st);
-        if (staged) {
+        if (P.staged) {
             k_fwh_geo<<<(int)(((long long)nb * nobs + 255) / 256), 256, 0, st>>>(
                 npts, j0, nb, d_xyz, d_area, d_obs, nobs, std::floor(t0 / dtau), 1.0 / c0, 1.0 / dtau, d_rec);
-            const dim3 go(ngroups, tb, nchunk);
-            const size_t sm = fwh_win_smem(W);
-            const bool full = nobs % FWH_MG == 0;
-            const auto launch = nth == 64    ? (full ? launch_obs_win<64, true> : launch_obs_win<64, false>)
-                                : nth == 128 ? (full ? launch_obs_win<128, true> : launch_obs_win<128, false>)
-                                             : (full ? launch_obs_win<256, true> : launch_obs_win<256, false>);
-            const int bad_attr = launch(go, sm, st, d_src, nb, N, d_rec, nobs, MG, t0, dt_obs, nt, T, dtau, chunk, W,
-                                        span, j0 > 0, d_part);
+            const dim3 go(P.ngroups, P.tblocks, nchunk);
+            const bool full = P.MG == FWH_MG && nobs % FWH_MG == 0;
+            const auto launch = P.nth == 64    ? (full ? launch_obs_win<64, true> : launch_obs_win<64, false>)
+                                : P.nth == 128 ? (full ? launch_obs_win<128, true> : launch_obs_win<128, false>)
+                                               : (full ? launch_obs_win<256, true> : launch_obs_win<256, false>);
+            const int bad_attr = launch(go, fwh_win_smem(P.W, fwh_rows(P.MG)), st, d_src, nb, N, d_rec, nobs, P.MG, t0,
+                                        dt_obs, nt, P.T, dtau, chunk, P.W, P.span, j0 > 0, d_part);
             if (bad_attr) rc = LES_ERR_CUDA;
         } else {
-            k_fwh_obs<<<dim3(tb, nobs, nchunk), FWH_T, 0, st>>>(d_src, npts, N, d_xyz, d_area, d_obs, nobs, t0, dt_obs,
-                                                               nt, dtau, c0, chunk, j0, nb, d_part);
+            k_fwh_obs<<<dim3(P.tblocks, nobs, nchunk), FWH_T, 0, st>>>(d_src, npts, N, d_xyz, d_area, d_obs, nobs, t0,
+                                                                      dt_obs, nt, dtau, c0, chunk, j0, nb, d_part);
         }
         if (cudaGetLastError() != cudaSuccess) rc = LES_ERR_CUDA;
         if (ms_out && rc == LES_OK) {

@@ -1,0 +1,51 @@
+"""The staged observer pass where a group's emission times spread over hundreds of frames, at the edges of what a
+window holds: short groups with a buffer row per microphone, blocks of 512 and of 256 times, full groups, and windows
+that leave the direct pass; against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import fwh
+from paper_2212_12365_gb300 import les
+from test_gpu_fwh import AMP, C0, P0, RHO0, SRC, _ring, _sphere
+
+pytestmark = pytest.mark.gpu
+DTAU, NFR = 0.02, 1700
+
+
+def _tone(xyz, w=2.5):
+    """Frames of a steadily sounding point monopole, which every microphone hears at any time."""
+    d = xyz - SRC[:, None]
+    R = np.sqrt((d * d).sum(axis=0))
+    tr = (DTAU * np.arange(NFR))[:, None] - R / C0
+    q, qd = AMP * np.sin(w * tr), AMP * w * np.cos(w * tr)
+    p = RHO0 * qd / (4 * np.pi * R)
+    u = (qd / (4 * np.pi * C0 * R) + q / (4 * np.pi * R * R))[:, None, :] * (d / R)
+    return np.concatenate([(RHO0 + p / C0 ** 2)[:, None], u, (P0 + p)[:, None]], axis=1)
+
+
+@pytest.fixture(scope="module")
+def data():
+    import torch
+    xyz, nrm, area = _sphere(1.0, 7, 13)
+    frames = _tone(xyz).astype(np.float32)
+    return xyz, nrm, area, frames.astype(np.float64), _ring(frames, NFR, torch.float32)
+
+
+# (microphones, times, spread of a group in frames, dt_obs / dtau)
+@pytest.mark.parametrize("mics,nt,spread,ratio", [
+    (2, 512, 480, 1.0), (3, 512, 640, 0.5), (7, 300, 640, 1.0), (8, 512, 470, 1.0), (9, 513, 380, 1.0),
+    (12, 512, 300, 1.0), (14, 512, 150, 1.0), (16, 512, 170, 1.0), (16, 512, 110, 1.0), (16, 257, 360, 1.0),
+    (16, 40, 560, 1.0), (16, 40, 700, 1.0), (32, 300, 200, 1.0), (40, 512, 260, 1.0)])
+def test_spread_groups(data, mics, nt, spread, ratio):
+    xyz, nrm, area, used, ring = data
+    # microphones along a ray; those of a group 16 (or fewer) apart cover the spread
+    far = 2.5 + C0 * DTAU * spread * np.arange(mics) / max(min(mics, 16) - 1, 1)
+    far = 2.5 + (far - 2.5) % (C0 * DTAU * spread + 1e-9)
+    obs = np.stack([0.8 * far, 0.5 * far, np.sqrt(1 - 0.89) * far])
+    t0 = (far.max() + 1.0) / C0 + 0.01
+    assert t0 + nt * ratio * DTAU - (far.min() - 1.0) / C0 < (NFR - 1) * DTAU
+    got = les.les_fwh(ring.data_ptr(), les.LES_FP32, NFR, NFR, xyz, nrm, area, DTAU, P0, C0, obs, t0, ratio * DTAU, nt)
+    ref = fwh.pressure(used, xyz, nrm, area, DTAU, RHO0, P0, C0, obs, t0, ratio * DTAU, nt)
+    # FP32 records and products: the bound of the other far-field tests, per microphone (each has its own distance)
+    scale = np.abs(ref).max(axis=1, keepdims=True)
+    assert (np.abs(got - ref) <= 2e-5 * scale).all(), (np.abs(got - ref) / scale).max(axis=1)
