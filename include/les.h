@@ -354,8 +354,10 @@ int les_measure_peak(int kind, double *tflops);
  * p_out: host, nobs*nt doubles, layout [observer][time]: p' = p - p0.
  * ms_out: NULL, or 2 doubles receiving the device time (ms) of the source
  *   pass and of the observer pass.
- * Allocates device scratch (32 bytes per panel and frame, plus partial sums)
- * for the call and frees it; runs on `stream`, synchronises it.  The sums
+ * Allocates device scratch for the call and frees it: 32 bytes per panel and
+ * frame and 32 per panel and observer, of as many panels at a time as keep
+ * each below 256 MB (the first: of 1024 panels if those take more), plus
+ * partial sums; runs on `stream`, synchronises it.  The sums
  * have a fixed order: the same inputs give the same bits.  Errors:
  * LES_ERR_ARG (null pointer, fewer than 3 frames, an emission time outside
  * the frames, an observer on a panel; text in les_last_error(NULL)),

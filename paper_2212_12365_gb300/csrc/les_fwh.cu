@@ -12,7 +12,9 @@
 // (one-sided three-point at the first and last frame), retarded values by
 // linear interpolation between the two frames around tau.
 //
-// Kernels, run over batches of panels whose source records take at most 256 MB:
+// Kernels, run over batches of panels whose source records, and whose records per
+// microphone, take at most 256 MB each (1024 panels' source records if those take
+// more):
 //   k_fwh_check : distances' range per microphone and the largest spread over
 //                 a microphone group (the input checks and the window length)
 //   k_fwh_src   : per panel and frame L, dQ/dtau and dL/dtau as two float4,

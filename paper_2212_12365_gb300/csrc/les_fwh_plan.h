@@ -77,8 +77,13 @@ inline FwhPlan fwh_plan(int npts, int N, int nobs, int nt, double dt_obs, double
     }
     // threads: half the block's times, so that few are idle in a short block
     P.nth = P.T <= 128 ? 64 : (P.T <= 256 ? 128 : 256);
-    // panels per batch: source records of at most 256 MB (and at least 1024 panels)
-    P.NB = (int)std::min<long long>(npts, std::max<long long>(1024, (256LL << 20) / (32LL * N) / 256 * 256));
+    // panels per batch: source records of at most 256 MB (and at least 1024
+    // panels, so that a batch fills the chip), and in the staged pass panel records
+    // of at most 256 MB too (from 8192 microphones on a batch has fewer than 1024
+    // panels, but the microphone groups alone fill the chip)
+    const long long batch = 256LL << 20;
+    P.NB = (int)std::min<long long>(npts, std::max<long long>(1024, batch / (32LL * N) / 256 * 256));
+    if (P.staged) P.NB = (int)std::min<long long>(P.NB, std::max<long long>(1, batch / (32LL * nobs)));
     // panel chunks of a batch: the CTAs of one wave (staged: 512 threads or the
     // shared memory of an SM; direct: four CTAs per SM)
     const int cps = P.staged ? std::min(512 / P.nth, (int)(2 * FWH_WIN_SMEM / fwh_win_smem(P.W, rows))) : 4;

@@ -82,3 +82,22 @@ def test_a_window_holds_its_block_and_fits_the_chip(plan):
         last = 1 + math.floor(spread) + 1 + math.floor((p["T"] - 1) * ratio + 1 + 1) + 1
         assert p["W"] % 32 == 0 and p["W"] <= 1024 and last <= p["W"] - 1 and p["span"] < p["W"]
         assert p["smem"] <= 110 * 1024 and p["nth"] >= (p["T"] + 1) // 2 and p["nth"] in (64, 128, 256)
+
+
+def test_scratch_is_bounded_by_the_records_of_a_batch(plan):
+    """Source records and panel records take at most 256 MB each, save where the source records of 1024 panels alone
+    take more; the records of the panels in hand are never more than those of all panels."""
+    rng = np.random.default_rng(3)
+    cases = [(98304, 64, 2048, 512, 1.0, 20.0), (98304, 3, 100000, 16, 1.0, 0.0), (2000000, 3, 64, 8, 1.0, 0.0)]
+    cases += [(int(2 ** rng.uniform(0, 21)), int(2 ** rng.uniform(1.6, 20)), int(2 ** rng.uniform(0, 18)),
+               int(2 ** rng.uniform(0, 12)), rng.uniform(0, 2), rng.uniform(0, 300)) for _ in range(4000)]
+    for npts, N, nobs, nt, ratio, spread in cases:
+        p = plan(npts, N, nobs, nt, ratio, spread * (nobs > 1))
+        assert p["b_src"] <= min(32 * npts * N, max(256 << 20, 32 * 1024 * N)), (npts, N, nobs)
+        assert p["b_rec"] <= max(256 << 20, 32 * nobs), (npts, N, nobs)
+        assert p["b_part"] <= 8 * nobs * nt * 1217
+
+
+def test_the_default_batch_keeps_its_panels(plan):
+    """Up to as many microphones as frames the batch is set by the source records alone."""
+    assert plan(98304, 1024, 64, 512, 1.0, 90)["NB"] == 8192

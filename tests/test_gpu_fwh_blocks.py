@@ -49,3 +49,22 @@ def test_spread_groups(data, mics, nt, spread, ratio):
     # FP32 records and products: the bound of the other far-field tests, per microphone (each has its own distance)
     scale = np.abs(ref).max(axis=1, keepdims=True)
     assert (np.abs(got - ref) <= 2e-5 * scale).all(), (np.abs(got - ref) / scale).max(axis=1)
+
+
+def test_many_microphones_in_several_batches():
+    """More (panel, microphone) records than one batch holds: the first microphones have the same pressure as in a
+    call of their own."""
+    import torch
+    xyz, nrm, area = _sphere(1.0, 23, 61)  # 1403 panels x 8192 microphones x 32 bytes: two batches
+    frames = _tone(xyz)[:300].astype(np.float32)
+    ring = _ring(frames, 300, torch.float32)
+    mics, nt = 8192, 5
+    a = np.linspace(0.1, 3.0, mics)
+    obs = np.stack([2.5 * np.cos(a), 2.5 * np.sin(a), 0.2 * np.sin(7 * a)])
+    t0 = 3.6 / C0 + 0.01
+    got = les.les_fwh(ring.data_ptr(), les.LES_FP32, 300, 300, xyz, nrm, area, DTAU, P0, C0, obs, t0, DTAU, nt)
+    few = les.les_fwh(ring.data_ptr(), les.LES_FP32, 300, 300, xyz, nrm, area, DTAU, P0, C0, obs[:, :160], t0, DTAU, nt)
+    ref = fwh.pressure(frames.astype(np.float64), xyz, nrm, area, DTAU, RHO0, P0, C0, obs[:, ::400], t0, DTAU, nt)
+    scale = np.abs(ref).max()
+    assert np.abs(got[::400] - ref).max() <= 2e-5 * scale
+    assert np.abs(got[:160] - few).max() <= 2e-6 * scale
