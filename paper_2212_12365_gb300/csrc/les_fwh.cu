@@ -91,12 +91,14 @@ __global__ void __launch_bounds__(128) k_fwh_src(const real *__restrict__ ring, 
 {
     typedef Num<real> A;
     typedef typename A::T T;
-    const int jl = blockIdx.x * blockDim.x + threadIdx.x;
+    // blocks: panels fastest, then segments (a grid's x alone holds any number)
+    const int pb = (nb + blockDim.x - 1) / blockDim.x, seg = blockIdx.x / pb;
+    const int jl = (blockIdx.x - seg * pb) * blockDim.x + threadIdx.x;
     if (jl >= nb) return;
     const int j = j0 + jl;
     const T n[3] = {A::of(nrm[j]), A::of(nrm[npts + j]), A::of(nrm[2 * npts + j])};
     const T mp0 = A::of(-p0), r2 = A::of(rdt2);
-    const int m0 = blockIdx.y * FWH_SEG, m1 = min(N, m0 + FWH_SEG);
+    const int m0 = seg * FWH_SEG, m1 = min(N, m0 + FWH_SEG);
     float4 *o = src + (long long)jl * N * 2;
     struct F {
         T v[4]; // L_x, L_y, L_z, Q
@@ -331,9 +333,11 @@ __global__ void __launch_bounds__(NTH, 512 / NTH) k_fwh_obs_win(const float4 *__
     float4 *RB = RA + W;                           // [W]: dL/dtau
     FwhGeo *G = (FwhGeo *)(RB + W);                // [FWH_PB]
     const int tid = threadIdx.x;
-    const int o0 = blockIdx.x * MG, mgt = FULL ? FWH_MG : min(MG, nobs - o0);
-    const int k0 = blockIdx.y * T, half = (min(T, nt - k0) + 1) / 2;
-    const int c = blockIdx.z;
+    // blocks: microphone groups fastest, then time blocks; panel chunks along y
+    const int ng = (nobs + MG - 1) / MG, tb = blockIdx.x / ng;
+    const int o0 = (blockIdx.x - tb * ng) * MG, mgt = FULL ? FWH_MG : min(MG, nobs - o0);
+    const int k0 = tb * T, half = (min(T, nt - k0) + 1) / 2;
+    const int c = blockIdx.y;
     // s(k) = t_k/dtau - B with B = floor of the block's first, an integer; split
     // into an integer and a fraction (a float of the whole offset would be good
     // to 3e-5 frames only)
@@ -576,7 +580,7 @@ extern "C" int les_fwh(const void *ring, int precision, int capacity, int64_t fr
         // the same chunk count in every batch; a short last batch has shorter chunks
         const int chunk = (nb + nchunk - 1) / nchunk;
         if (ms_out) cudaEventRecord(ev[0], st);
-        const dim3 gs((nb + 127) / 128, (N + FWH_SEG - 1) / FWH_SEG);
+        const int gs = (nb + 127) / 128 * ((N + FWH_SEG - 1) / FWH_SEG);
         if (precision == LES_FP64)
             k_fwh_src<double><<<gs, 128, 0, st>>>((const double *)ring, first, capacity, npts, j0, nb, N, d_nrm, p0,
                                                   rdt2, d_src);
@@ -587,7 +591,7 @@ extern "C" int les_fwh(const void *ring, int precision, int capacity, int64_t fr
         if (P.staged) {
             k_fwh_geo<<<(int)(((long long)nb * nobs + 255) / 256), 256, 0, st>>>(
                 npts, j0, nb, d_xyz, d_area, d_obs, nobs, std::floor(t0 / dtau), 1.0 / c0, 1.0 / dtau, d_rec);
-            const dim3 go(P.ngroups, P.tblocks, nchunk);
+            const dim3 go(P.ngroups * P.tblocks, nchunk);
             const bool full = P.MG == FWH_MG && nobs % FWH_MG == 0;
             const auto launch = P.nth == 64    ? (full ? launch_obs_win<64, true> : launch_obs_win<64, false>)
                                 : P.nth == 128 ? (full ? launch_obs_win<128, true> : launch_obs_win<128, false>)

@@ -68,3 +68,51 @@ def test_many_microphones_in_several_batches():
     scale = np.abs(ref).max()
     assert np.abs(got[::400] - ref).max() <= 2e-5 * scale
     assert np.abs(got[:160] - few).max() <= 2e-6 * scale
+
+
+def _line(n_frames, panels=1):
+    """A ring of a slow tone at a panel (or a few), made on the GPU, with a period of 400 frames."""
+    import torch
+    t = (torch.arange(n_frames, device="cuda") % 400).double() * (2 * np.pi / 400)
+    ring = torch.empty((n_frames, 5, panels), dtype=torch.float32, device="cuda")
+    for f, (mean, amp, ph) in enumerate(((RHO0, 1e-2, 0.0), (0.0, 2e-2, 0.4), (0.0, 1e-2, 1.1), (0.0, 0.0, 0.0), (P0, 1e-2, 2.0))):
+        ring[:, f] = (mean + amp * torch.sin(t + ph)).float()[:, None]
+    return ring
+
+
+def _panel(panels=1):
+    xyz = np.zeros((3, panels))
+    xyz[0] = 0.01 * np.arange(panels)
+    nrm = np.tile(np.array([[1.0], [0.0], [0.0]]), (1, panels))
+    return xyz, nrm, np.full(panels, 0.3)
+
+
+def test_more_frames_than_a_grid_has_rows():
+    """4.2 million frames: the source pass covers them all (65,535 segments of 64 frames and more)."""
+    n = 65535 * 64 + 1000
+    xyz, nrm, area = _panel()
+    ring = _line(n)
+    obs = np.array([[3.0, 1.0, 0.5]]).T
+    # the last 300 observer times that the frames cover; the tone repeats every 400 frames, so the same times of a
+    # ring of 2000 frames (a whole number of periods earlier) give the same pressure
+    shift = (n - 2000) // 400 * 400
+    t_short = 1600 * DTAU
+    args = (xyz, nrm, area, DTAU, P0, C0, obs)
+    got = les.les_fwh(ring.data_ptr(), les.LES_FP32, n, n, *args, t_short + shift * DTAU, DTAU, 300)
+    ref = les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, *args, t_short, DTAU, 300)
+    assert np.abs(ref).max() > 0 and np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
+def test_more_time_blocks_than_a_grid_has_rows():
+    """34 million observer times: more than 65,535 blocks of 512."""
+    nt = 65535 * 512 + 700
+    xyz, nrm, area = _panel(3)
+    ring = _line(2000, 3)
+    obs = np.array([[3.0, 1.0, 0.5]]).T
+    t0, dt_obs = 5.0, 30.0 / nt
+    args = (xyz, nrm, area, DTAU, P0, C0, obs)
+    got = les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, *args, t0, dt_obs, nt)[0]
+    ref = les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, *args, t0 + (nt - 500) * dt_obs, dt_obs, 500)[0]
+    assert np.abs(got[-500:] - ref).max() <= 1e-5 * np.abs(ref).max()
+    every = les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, *args, t0, dt_obs * 65536, nt // 65536)[0]
+    assert np.abs(got[::65536][:every.size] - every).max() <= 1e-5 * np.abs(every).max()
