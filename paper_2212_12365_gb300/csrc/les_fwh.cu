@@ -465,8 +465,10 @@ static int launch_obs_win(dim3 grid, size_t smem, cudaStream_t st, const float4 
                           int nobs, int MG, double t0, double dt_obs, int nt, int T, double dtau, int chunk, int W,
                           int span, int add, double *part)
 {
-    if (cudaFuncSetAttribute(k_fwh_obs_win<NTH, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    // always the same limit: it belongs to the kernel, and calls from other host
+    // threads may need another size between this line and the launch
+    if (cudaFuncSetAttribute(k_fwh_obs_win<NTH, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)FWH_WIN_SMEM) != cudaSuccess)
         return 1;
     k_fwh_obs_win<NTH, FULL><<<grid, NTH, smem, st>>>(src, nb, N, geo, nobs, MG, t0, dt_obs, nt, T, dtau, chunk, W,
                                                       span, add, part);

@@ -116,3 +116,30 @@ def test_more_time_blocks_than_a_grid_has_rows():
     assert np.abs(got[-500:] - ref).max() <= 1e-5 * np.abs(ref).max()
     every = les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, *args, t0, dt_obs * 65536, nt // 65536)[0]
     assert np.abs(got[::65536][:every.size] - every).max() <= 1e-5 * np.abs(every).max()
+
+
+def test_two_threads_with_windows_of_different_size():
+    """Calls from two host threads whose staged passes need different amounts of shared memory."""
+    import threading
+    import torch
+    xyz, nrm, area = _panel(64)
+    ring = _line(2000, 64)
+    obs = np.array([[3.0, 1.0, 0.5], [2.0, -1.0, 0.5]]).T
+    torch.cuda.synchronize()
+    errors = []
+
+    def calls(ratio):
+        try:
+            st = torch.cuda.Stream()
+            for _ in range(1500):
+                les.les_fwh(ring.data_ptr(), les.LES_FP32, 2000, 2000, xyz, nrm, area, DTAU, P0, C0, obs, 6.0,
+                            ratio * DTAU, 512, stream=st.cuda_stream)
+        except Exception as e:  # noqa: BLE001 (handed to the test's thread)
+            errors.append(e)
+
+    th = [threading.Thread(target=calls, args=(r,)) for r in (0.05, 1.0)]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not errors, errors
