@@ -542,6 +542,29 @@ static std::string kc_label(int kc)
 }
 static int autotune_fused(les_handle *h);
 
+// Optional event timing around every launch (les_profile_step); inactive during capture.
+struct Tracer {
+    cudaStream_t st = nullptr; // may be the legacy default stream (NULL)
+    std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev;
+    void begin(int kind)
+    {
+        cudaEvent_t a, b;
+        cudaEventCreate(&a);
+        cudaEventCreate(&b);
+        cudaEventRecord(a, st);
+        ev.push_back({kind, {a, b}});
+    }
+    void end() { cudaEventRecord(ev.back().second.second, st); }
+};
+// One kernel launch of the given kind, timed if a tracer is there; counts 1.
+template <typename F> static int traced(Tracer *tr, int kind, const F &launch)
+{
+    if (tr) tr->begin(kind);
+    launch();
+    if (tr) tr->end();
+    return 1;
+}
+
 // One form's launch of a fused stage (or residual) over all its jets (jet < 0)
 // or one jet.
 static void fused_launch_form(les_handle *h, int fi, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st)
@@ -567,14 +590,13 @@ static void fused_launch_form(les_handle *h, int fi, int jet, int src, int dst, 
 }
 
 // The same for every form in use; returns the number of launches.
-static int fused_launch(les_handle *h, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st)
+static int fused_launch(les_handle *h, int jet, int src, int dst, int stage, int rhs_only, cudaStream_t st,
+                        Tracer *tr = nullptr)
 {
     int n = 0;
     for (int fi = 0; fi < 2; ++fi)
-        if (jet < 0 ? h->form[fi].any : form_of(h, jet) == fi) {
-            fused_launch_form(h, fi, jet, src, dst, stage, rhs_only, st);
-            ++n;
-        }
+        if (jet < 0 ? h->form[fi].any : form_of(h, jet) == fi) // counted as the interface kernel kind
+            n += traced(tr, LES_KERNEL_IFACE, [&] { fused_launch_form(h, fi, jet, src, dst, stage, rhs_only, st); });
     return n;
 }
 
@@ -871,100 +893,64 @@ template <typename real> static const JetDev<real> *only_jet(const les_handle *h
 // One part (0 point, 1 gradients, 2 interfaces, 3 update) of the FP64 stage over
 // all jets (jet < 0) or one: the jets of the general form, then those of the
 // product form.  Returns the number of launches.
-static int fp64_part(les_handle *h, int jet, int part, int src, int dst, int stage, int rhs_only, cudaStream_t st)
+static int fp64_part(les_handle *h, int jet, int part, int src, int dst, int stage, int rhs_only, cudaStream_t st,
+                     Tracer *tr = nullptr)
 {
+    int n = 0;
     const JetDev<double> *jets = (const JetDev<double> *)h->d_jets + (jet < 0 ? 0 : jet);
     const BlockMap &g = jet < 0 ? h->ptg : h->ptg1[jet], &p = jet < 0 ? h->ptp : h->ptp1[jet];
     const double *dt = h->d_dt + (jet < 0 ? 0 : jet);
     if (g.total > 0) {
         const int gp = grid_cap(h, g.total);
-        switch (part) {
-        case 0: Launch<double>::point(jets, g, src, gp, st); break;
-        case 1: Launch<double>::grads(jets, g, gp, st); break;
-        case 2: Launch<double>::iface(jets, g, gp, st); break;
-        default: Launch<double>::update(jets, g, dst, stage, dt, rhs_only, gp, st); break;
-        }
+        n += traced(tr, LES_KERNEL_POINT + part, [&] {
+            switch (part) {
+            case 0: Launch<double>::point(jets, g, src, gp, st); break;
+            case 1: Launch<double>::grads(jets, g, gp, st); break;
+            case 2: Launch<double>::iface(jets, g, gp, st); break;
+            default: Launch<double>::update(jets, g, dst, stage, dt, rhs_only, gp, st); break;
+            }
+        });
     }
     // one block per 64 points: the hardware balances them over the SMs
-    if (p.total > 0) launch_stage_prod(jets, p, part, src, dst, stage, dt, rhs_only, p.total, st);
-    return (g.total > 0) + (p.total > 0);
+    if (p.total > 0)
+        n += traced(tr, LES_KERNEL_POINT + part,
+                    [&] { launch_stage_prod(jets, p, part, src, dst, stage, dt, rhs_only, p.total, st); });
+    return n;
 }
 
 // Boundary conditions of the current level on all jets (jet < 0) or one;
 // returns the number of launches.
-template <typename real> static int bc_pass(les_handle *h, int jet, int dst, cudaStream_t st)
+template <typename real> static int bc_pass(les_handle *h, int jet, int dst, cudaStream_t st, Tracer *tr = nullptr)
 {
     const JetDev<real> *jets = (const JetDev<real> *)h->d_jets + (jet < 0 ? 0 : jet);
     const BlockMap &bm = jet < 0 ? h->bcm : h->bc1[jet];
-    if (h->centerline) launch_centerline<real>(jets, bm.njets, h->max_ni, dst, st);
-    Launch<real>::bc(jets, bm, dst, h->d_level, only_jet<real>(h, jet), st);
-    return (h->centerline ? 1 : 0) + (bm.total > 0 ? 1 : 0);
+    int n = 0;
+    if (h->centerline)
+        n += traced(tr, LES_KERNEL_BC, [&] { launch_centerline<real>(jets, bm.njets, h->max_ni, dst, st); });
+    if (bm.total > 0) // none on a fully periodic grid
+        n += traced(tr, LES_KERNEL_BC,
+                    [&] { Launch<real>::bc(jets, bm, dst, h->d_level, only_jet<real>(h, jet), st); });
+    return n;
 }
-
-// Optional per-launch event timing (les_profile_step); inactive during capture.
-struct Tracer {
-    bool on = false;
-    cudaStream_t st = nullptr; // may be the legacy default stream (NULL)
-    std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev;
-    void begin(int kind)
-    {
-        if (!on) return;
-        cudaEvent_t a, b;
-        cudaEventCreate(&a);
-        cudaEventCreate(&b);
-        cudaEventRecord(a, st);
-        ev.push_back({kind, {a, b}});
-    }
-    void end()
-    {
-        if (!on) return;
-        cudaEventRecord(ev.back().second.second, st);
-    }
-};
 
 template <typename real> static int record_step(les_handle *h, cudaStream_t st, Tracer *tr = nullptr)
 {
-    Tracer none;
-    Tracer &T = tr ? *tr : none;
     const JetDev<real> *jets = (const JetDev<real> *)h->d_jets;
     static const int src_of[5] = {0, 1, 2, 1, 2};
     static const int dst_of[5] = {1, 2, 1, 2, 0};
-    h->launches_per_step = 0;
-    T.begin(LES_KERNEL_OTHER);
-    launch_step_advance(h->d_level, st);
-    T.end();
-    h->launches_per_step++;
+    int64_t n = traced(tr, LES_KERNEL_OTHER, [&] { launch_step_advance(h->d_level, st); });
     for (int s = 0; s < 5; ++s) {
-        if (h->prec == LES_FP32) {
-            // fused single-pass stage: counted as the interface kernel kind
-            T.begin(LES_KERNEL_IFACE);
-            h->launches_per_step += fused_launch(h, -1, src_of[s], dst_of[s], s, 0, st);
-            T.end();
-            if (h->bcm.total > 0) { // none on a fully periodic grid
-                T.begin(LES_KERNEL_BC);
-                h->launches_per_step += bc_pass<real>(h, -1, dst_of[s], st);
-                T.end();
-            }
-            continue;
-        }
-        for (int part = 0; part < 4; ++part) {
-            T.begin(LES_KERNEL_POINT + part);
-            h->launches_per_step += fp64_part(h, -1, part, src_of[s], dst_of[s], s, 0, st);
-            T.end();
-        }
-        if (h->bcm.total > 0) { // none on a fully periodic grid
-            T.begin(LES_KERNEL_BC);
-            h->launches_per_step += bc_pass<real>(h, -1, dst_of[s], st);
-            T.end();
-        }
+        if (h->prec == LES_FP32) n += fused_launch(h, -1, src_of[s], dst_of[s], s, 0, st, tr);
+        else
+            for (int part = 0; part < 4; ++part) n += fp64_part(h, -1, part, src_of[s], dst_of[s], s, 0, st, tr);
+        n += bc_pass<real>(h, -1, dst_of[s], st, tr);
     }
-    if (h->probe_npts > 0) {
-        T.begin(LES_KERNEL_OTHER);
-        Launch<real>::probe(jets, h->d_cell, h->d_wts, h->probe_npts, h->probe_every, h->d_level,
-                            h->d_probe_base, (real *)h->probe_out, h->probe_cap, st);
-        T.end();
-        h->launches_per_step++;
-    }
+    if (h->probe_npts > 0)
+        n += traced(tr, LES_KERNEL_OTHER, [&] {
+            Launch<real>::probe(jets, h->d_cell, h->d_wts, h->probe_npts, h->probe_every, h->d_level, h->d_probe_base,
+                                (real *)h->probe_out, h->probe_cap, st);
+        });
+    h->launches_per_step = n;
     CK(cudaGetLastError());
     return LES_OK;
 }
@@ -977,7 +963,6 @@ template <typename real> static int profile_impl(les_handle *h, int nsteps, doub
     }
     for (int s = 0; s < nsteps; ++s) {
         Tracer tr;
-        tr.on = true;
         tr.st = h->st;
         int rc = record_step<real>(h, h->st, &tr);
         CK(cudaStreamSynchronize(h->st));
