@@ -1327,11 +1327,13 @@ extern "C" int les_set_fused_tiling(les_handle *h, int ty, int kc)
 {
     if (!h) return LES_ERR_ARG;
     if (h->prec != LES_FP32) return fail(h, LES_ERR_ARG, "the fused tiling applies to FP32 handles");
-    if ((ty != 8 && ty != 16) || kc < -1) return fail(h, LES_ERR_ARG, "ty must be 8 or 16 and kc >= -1");
+    if ((ty != 8 && ty != 16 && !(ty == 24 && h->form[1].any)) || kc < -1)
+        return fail(h, LES_ERR_ARG, "ty must be 8, 16 or, for jets on product grids, 24, and kc >= -1");
     for (int fi = 0; fi < 2; ++fi) {
-        int rc = set_fused_tiling(h, fi, ty, kc);
+        const int t = fi == 0 ? std::min(ty, 16) : ty; // 24 rows: product form only
+        int rc = set_fused_tiling(h, fi, t, kc);
         if (rc) return rc;
-        h->form[fi].note = "ty=" + std::to_string(ty) + " kc=" + kc_label(kc) + " (set by the caller)";
+        h->form[fi].note = "ty=" + std::to_string(t) + " kc=" + kc_label(kc) + " (set by the caller)";
     }
     h->tuned = true;
     if (h->gexec) { // the captured step holds the old work list
