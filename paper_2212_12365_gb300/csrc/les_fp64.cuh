@@ -1,13 +1,18 @@
 // FP64 building blocks of the stage kernels, chosen to issue few FP64
 // instructions: GB300's FP64 pipe takes two lanes per clock and SM.
 //
-// Reciprocals and square roots iterate from the hardware's approximate seeds
-// (about 20 bits).  With e = 1 - b y0, the series 1/b = y0 (1 + e + e^2 + ...)
-// cut after e^2 leaves e^3 ~ 2^-60: three operations (two Newton steps take
-// four).  For the square root, with t = x y0, e = 1 - t y0, sqrt(x) =
-// t (1 + e/2 + 3 e^2/8 + ...): five operations, against eight of the
-// library's sqrt; both round to within about an ulp.  Comparisons of
-// non-negative numbers go to the integer pipe.
+// Reciprocals and square roots refine the hardware's approximate seeds (about 20
+// bits) by one step of a power series in the seed's error.  With e = 1 - b y0
+// (exact to 2^-73 by the fused multiply-add), 1/b = y0 (1 + e + e^2 + ...) cut
+// after e^2 leaves e^3 ~ 2^-60: three operations.  With e = 1 - x y0^2, the
+// binomial series (1 - e)^(-1/2) = 1 + e/2 + 3 e^2/8 + ... cut after e^2 gives
+// x^(-1/2), within about an ulp.  The square root takes the same series on the
+// residual: t = x y0 rounded, r = x - t^2 (exact but for its last bit), sqrt(x) =
+// t + r y0 (1/2 + 3 e/8), so that the rounding of t does not reach the result:
+// six operations, within 0.53 ulp.  (As t (1 + e/2 + 3 e^2/8), five operations,
+// it was off by up to 0.76 ulp; ten FP64 steps took 3116 us on 48x32x32 and 34.05
+// ms on the polar 200x75x40 with that form and take 3144 us and 34.32 ms.)
+// Comparisons of non-negative numbers go to the integer pipe.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -47,16 +52,21 @@ __device__ __forceinline__ double rsqrt64(double x)
     const double e = fma(-(x * y), y, 1.0);
     return fma(y, e * fma(0.375, e, 0.5), y);
 }
-// x^1/2, x >= 0; 0 below the normal range
-template <int E> // times 2^E
-__device__ __forceinline__ double sqrt64_scaled(double x)
+// y 2^E, y and the result normal
+template <int E> __device__ __forceinline__ double scaled64(double y)
 {
-    const double y = rsqrt_seed64(x);
-    const double t0 = x * y;
-    const double e = fma(-t0, y, 1.0);
-    const double t = E != 0 ? __hiloint2double(__double2hiint(t0) + E * (1 << 20), __double2loint(t0)) : t0;
-    const double s = fma(t, e * fma(0.375, e, 0.5), t);
-    return __double2hiint(x) < 0x00100000 && __double2hiint(x) >= 0 ? 0.0 : s;
+    return E != 0 ? __hiloint2double(__double2hiint(y) + E * (1 << 20), __double2loint(y)) : y;
+}
+// x^1/2 times 2^E, x >= 0; 0 below the normal range, infinity from infinity (and
+// NaN from x < 0)
+template <int E> __device__ __forceinline__ double sqrt64_scaled(double x)
+{
+    const double y = rsqrt_seed64(x), t = x * y;
+    const double e = fma(-t, y, 1.0), r = fma(-t, t, x);
+    const double s = fma(r * scaled64<E>(y), fma(0.375, e, 0.5), scaled64<E>(t));
+    const int h = __double2hiint(x), m = h & 0x7fffffff;
+    if (m < 0x00100000) return 0.0;
+    return h == 0x7ff00000 ? x : s; // (NaN stays NaN: s is one)
 }
 __device__ __forceinline__ double sqrt64(double x) { return sqrt64_scaled<0>(x); }
 __device__ __forceinline__ double twice_sqrt64(double x) { return sqrt64_scaled<1>(x); }
