@@ -7,13 +7,14 @@
 // six FP64 operations, and GB300's FP64 pipe (2 lanes per clock and SM) takes
 // 1.4 ms for five of them per point: the pipe, not memory, bounded the sums.
 // So the conservation sums run on the integer pipe: every lane keeps a 128-bit
-// fixed-point sum (SumFx) whose least bit sits 2^-44 below the last bit of the
-// largest value its warp has met; the additions are exact above that bit.  The
-// truncated tails are below 2^-96 of the largest value each, so the sum is as
-// good as the compensated one (a test holds both to the exactly rounded sum).
+// fixed-point sum (SumFx) whose least bit sits 2^-52 below the last bit of the
+// largest value its warp has met; the additions are exact above that bit, and
+// what reaches below it is kept in a double of its own, so that large values may
+// cancel without a trace (a test holds the sums to the exactly rounded ones).
 // The sums of squares stay in FP64 (one multiply-add per value).
-// Measured: 14,155,776 points 2098 -> 236 us (4.8 TB/s); les_get_diagnostics of
-// a 192x128x72 FP32 jet about 1.0 ms less per call (most of it the final pass).
+// Measured: 14,155,776 points 2098 -> 244 us (4.6 TB/s; 236 without the tails);
+// les_get_diagnostics of a 192x128x72 FP32 jet about 1.0 ms less per call (most of
+// it the final pass).
 #pragma once
 
 #include "les_internal.cuh"
@@ -45,43 +46,64 @@ __device__ __forceinline__ double scale2(double x, int k)
     return ldexp(ldexp(x, h), k - h);
 }
 
-// Fixed-point sum of doubles: value = (hi 2^64 + lo) 2^(base - 1075), the
-// base (a biased exponent) the same for all lanes of a warp.
+// Fixed-point sum of doubles: value = (hi 2^64 + lo) 2^(base - 1075) + the
+// lane's tail, the base (a biased exponent) the same for all lanes of a warp.
+// Bits below the base go to the tail, a double: its terms are below one unit of
+// the base each, so that its rounding is some 2^-150 of the largest value.
 struct SumFx {
     long long hi = 0;
     unsigned long long lo = 0;
     int base = -4096; // below every exponent: the first value sets it
 
-    static constexpr int GUARD = 44; // bits kept below the largest value's last bit
+    static constexpr int GUARD = 52; // bits kept below the largest value's last bit
     static constexpr int TOP = 55;   // largest shift: 53 + 55 bits, 19 bits left for the count and sign
 
     // Add a finite v; every lane of the warp calls it together.
-    __device__ __forceinline__ void add(double v)
+    __device__ __forceinline__ void add(double v, double *tail)
     {
         const long long b = __double_as_longlong(v);
         const int ef = (int)((unsigned long long)b >> 52) & 0x7ff;
-        const int e = max(ef, 1); // subnormals have no hidden bit and exponent 1
+        int e = max(ef, 1); // subnormals have no hidden bit and exponent 1
         long long m = (b & 0xFFFFFFFFFFFFFll) | (ef ? 1ll << 52 : 0ll);
+        // a value above the window, or reaching below it (seldom: within 2^-52 of
+        // the largest value so far there is none)
+        if (__any_sync(0xffffffffu, m != 0 && (unsigned)(e - base) > (unsigned)TOP)) {
+            const int top = __reduce_max_sync(0xffffffffu, m != 0 ? e : -4096);
+            if (top - base > TOP) rebase(top - GUARD, tail);
+            const int d = base - e;
+            if (m != 0 && d > 0) { // the lowest d bits
+                const long long low = d > 52 ? ~0ll : (1ll << d) - 1;
+                *tail += v - (d > 52 ? 0.0 : __longlong_as_double(b & ~low));
+                m = d > 52 ? 0 : m >> d;
+                e = base;
+            }
+        }
         m = b < 0 ? -m : m;
-        if (__any_sync(0xffffffffu, e - base > TOP)) rebase(__reduce_max_sync(0xffffffffu, e) - GUARD);
-        const int s = e - base;
-        m >>= min(max(-s, 0), 63);
-        const int l = max(s, 0);
+        const int l = (e - base) & 63;
         const unsigned long long al = (unsigned long long)m << l;
         const long long ah = (m >> 1) >> (63 - l);
         lo += al;
         hi += ah + (lo < al ? 1 : 0);
     }
-    // Move the least bit up: what falls off is below 2^-96 of the new largest value.
-    __device__ __forceinline__ void rebase(int nb)
+    // Move the least bit up; what falls off goes to the tail.
+    __device__ __forceinline__ void rebase(int nb, double *tail)
     {
-        const int d = min(nb - base, 127);
-        if (d >= 64) {
-            lo = (unsigned long long)(hi >> (d - 64));
-            hi >>= 63;
-        } else if (d > 0) {
-            lo = (lo >> d) | ((unsigned long long)hi << (64 - d));
-            hi >>= d;
+        const int d = nb - base;
+        if ((hi | (long long)lo) != 0) {
+            const int u = base - 1075;
+            if (d >= 120) { // less than a few units of the new base
+                *tail += scale2((double)hi, u + 64) + scale2((double)lo, u);
+                hi = 0;
+                lo = 0;
+            } else if (d >= 64) {
+                *tail += scale2((double)(hi & ((1ll << (d - 64)) - 1)), u + 64) + scale2((double)lo, u);
+                lo = (unsigned long long)(hi >> (d - 64));
+                hi >>= 63;
+            } else {
+                *tail += scale2((double)(lo & ((1ull << d) - 1)), u);
+                lo = (lo >> d) | ((unsigned long long)hi << (64 - d));
+                hi >>= d;
+            }
         }
         base = nb;
     }
@@ -115,6 +137,11 @@ struct SumFx {
 template <typename Load> __device__ __forceinline__ void sum_block(long long steps, const Load &load, double *part)
 {
     SumFx fx[5];
+    // the lanes' tails: in shared memory, since they are seldom touched and the
+    // registers hold the next point
+    __shared__ double tails[5][SUM_BLOCK];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) tails[f][threadIdx.x] = 0.0;
     double l2[5] = {0, 0, 0, 0, 0};
     long long mxb = 0; // |RHS_rho| as its bits, which order as integers (NaN ignored, as fmax does)
     int bad = 0;
@@ -138,7 +165,7 @@ template <typename Load> __device__ __forceinline__ void sum_block(long long ste
             bad += !(vf && rf);
             if (!vf) nf |= 1u << f;
             l2[f] = fma(r[f], r[f], l2[f]);
-            fx[f].add(vf ? q[f] : 0.0);
+            fx[f].add(vf ? q[f] : 0.0, &tails[f][threadIdx.x]);
         }
     }
     __shared__ double sh[SUM_PART][SUM_BLOCK / 32];
@@ -155,9 +182,13 @@ template <typename Load> __device__ __forceinline__ void sum_block(long long ste
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
         fx[f].warp_reduce();
+        double tail = tails[f][threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
         if (lane == f) {
             double s, c;
             fx[f].value(s, c);
+            c += tail;
             sh[1 + f][w] = l2[f];
             sh[6 + f][w] = (nf >> f) & 1 ? __longlong_as_double(0x7ff8000000000000ll) : s;
             sh[11 + f][w] = c;
