@@ -40,28 +40,6 @@ namespace {
 
 constexpr int FWH_SUB = 256; // panels per shared-memory sub-chunk
 
-// Ring frame m (0 = oldest used) of field f at panel j.
-template <typename real>
-__device__ __forceinline__ double ring_at(const real *ring, int first, int cap, int npts, int m, int f, int j)
-{
-    const int slot = (first + m) % cap;
-    return (double)ring[((long long)slot * 5 + f) * npts + j];
-}
-
-// Q and L of panel j at ring frame m.
-template <typename real>
-__device__ __forceinline__ void ql_at(const real *ring, int first, int cap, int npts, int m, int j, const double n[3],
-                                      double p0, double &Q, double L[3])
-{
-    const double rho = ring_at(ring, first, cap, npts, m, 0, j);
-    const double u[3] = {ring_at(ring, first, cap, npts, m, 1, j), ring_at(ring, first, cap, npts, m, 2, j),
-                         ring_at(ring, first, cap, npts, m, 3, j)};
-    const double p = ring_at(ring, first, cap, npts, m, 4, j);
-    const double un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
-    Q = rho * un;
-    for (int i = 0; i < 3; ++i) L[i] = (p - p0) * n[i] + rho * u[i] * un;
-}
-
 // 32-byte store (16-byte halves a, b) to a 32-byte aligned address
 __device__ __forceinline__ void store8(float4 *p, const float4 &a, const float4 &b)
 {
