@@ -286,63 +286,9 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
     if (tid == 0) mbar_init(S.MBAR);
     __syncthreads();
 
-    // Work cursor: items (jet, tile, k-chunk) strided over the grid
-    // (balanced = 0), or the CTA's contiguous, equal share of all tile-planes
-    // (jet-major, tile, then plane), cut into one column piece per tile it
-    // touches (balanced = 1).  balanced = 2 (lockstep) first runs
-    // total_tiles / gridDim.x waves of whole columns (tile blockIdx.x +
-    // wave * gridDim.x: the CTAs march k together, so neighbouring tiles read
-    // their shared halo planes within a short window, mostly from L2) and
-    // shares out the remaining tile-planes the same way.  A piece starting
-    // mid-column recomputes its first zeta flux, so the result does not
-    // depend on where the cuts fall.
-    int item = blockIdx.x, w = 0, wend = 0;
-    const int nwave = balanced == 2 ? total_tiles / (int)gridDim.x : 0;
-    int wave = 0;
-    auto jet_of_tile = [&](int t) {
-        if constexpr (ONE) return 0;
-        int lo = 0, hi = njets;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (fj[mid].tile0 <= t) lo = mid; else hi = mid;
-        }
-        return lo;
-    };
-    auto next_range = [&]() {
-        while (wave <= nwave) {
-            if (wave < nwave) {
-                const int t = blockIdx.x + wave * gridDim.x;
-                const FusedJet &Fw = jet_entry<ONE>(f1, fj, jet_of_tile(t));
-                w = Fw.item0 + (t - Fw.tile0) * Fw.nkc;
-                wend = w + Fw.nkc;
-            } else {
-                const int t1 = nwave * gridDim.x;
-                int i1 = total_items;
-                if (t1 < total_tiles) {
-                    const FusedJet &Fw = jet_entry<ONE>(f1, fj, jet_of_tile(t1));
-                    i1 = Fw.item0 + (t1 - Fw.tile0) * Fw.nkc;
-                }
-                const long long rem = total_items - i1;
-                w = i1 + (int)((rem * blockIdx.x) / gridDim.x);
-                wend = i1 + (int)((rem * (blockIdx.x + 1)) / gridDim.x);
-            }
-            ++wave;
-            if (w < wend) return true;
-        }
-        return false;
-    };
-    if (balanced) next_range();
-    while (balanced ? (w < wend || next_range()) : item < total_items) {
-        const int key = balanced ? w : item;
-        int jet = 0;
-        if constexpr (!ONE) {
-            int lo = 0, hi = njets;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (fj[mid].item0 <= key) lo = mid; else hi = mid;
-            }
-            jet = lo;
-        }
+    Cursor<ONE> cur(fj, f1, njets, total_items, total_tiles, balanced);
+    int key, jet;
+    while (cur.next(key, jet)) {
         const JetDev<float> &J = jet_entry<ONE>(j1, jets, jet);
         const FusedJet &F = jet_entry<ONE>(f1, fj, jet);
         if constexpr (!ONE) {
@@ -360,25 +306,7 @@ __global__ void __launch_bounds__(FX * TY / 2, 1)
         const int jlo = 1, jhi = pj ? nj + 1 : nj - 1;
         const int klo = pk ? 0 : 1, khi = pk ? nk : nk - 1;
         int bx, by, k0, k1;
-        if (balanced) {
-            const int np = khi - klo; // planes per column (F.nkc)
-            const int r = key - F.item0;
-            const int tile = r / np, pl = r - tile * np;
-            bx = tile % F.nbx;
-            by = tile / F.nbx;
-            k0 = klo + pl;
-            k1 = klo + min(np, pl + (wend - w));
-            w += k1 - k0;
-        } else {
-            int r = key - F.item0;
-            bx = r % F.nbx;
-            r /= F.nbx;
-            by = r % F.nby;
-            const int kc = r / F.nby;
-            k0 = klo + kc * F.kc;
-            k1 = min(k0 + F.kc, khi);
-            item += gridDim.x;
-        }
+        cur.take(key, F, klo, khi, bx, by, k0, k1);
         const int i0 = ilo + bx * (FX - 2), j0 = jlo + by * (TY - 2);
         const int ib = i0 - 1, jb = j0 - 1; // grid column / row of the tile's first R1 cell (jb even)
         // 32-bit offsets: creation limits an FP32 jet to 5 fields x fs and its
