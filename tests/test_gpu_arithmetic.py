@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2212_12365_gb300", "csrc")
 SRC = r"""
 #include "les_fp64.cuh"
+#include "les_bc.cuh"
 #include "les_fused.cuh"
 #include "les_pair.cuh"
 using namespace les;
@@ -43,11 +44,25 @@ __global__ void kpair(const float *a, const float *b, int n, float *o) // a, b: 
         o[(2 * f + 1) * n + i] = v[f].l;
     }
 }
+// energy_pair of a state at rest but for rho u: 1/rho, and the internal energy
+__global__ void kenergy(const float *q, int n, float *o)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float Q[5] = {q[i], q[n + i], q[2 * n + i], q[3 * n + i], q[4 * n + i]};
+    FloatPair rr, ei;
+    energy_pair(Q, rr, ei);
+    o[i] = rr.h;
+    o[n + i] = rr.l;
+    o[2 * n + i] = ei.h;
+    o[3 * n + i] = ei.l;
+}
 extern "C" int run(int which, const void *a, const void *b, int n, void *o)
 {
     const int g = (n + 255) / 256;
     if (which == 0) k64<<<g, 256>>>((const double *)a, n, (double *)o);
     else if (which == 1) k32<<<g, 256>>>((const float *)a, n, (float *)o);
+    else if (which == 3) kenergy<<<g, 256>>>((const float *)a, n, (float *)o);
     else kpair<<<g, 256>>>((const float *)a, (const float *)b, n, (float *)o);
     return cudaDeviceSynchronize() != cudaSuccess;
 }
@@ -144,3 +159,16 @@ def test_pairs_of_floats(run):
     for f, (exact, scale) in enumerate(((A + B, abs(A) + abs(B)), (A - B, abs(A) + abs(B)), (A * B, abs(A * B)), (a0 * B, abs(a0 * B)))):
         rel = np.abs((v[2 * f] + v[2 * f + 1] - exact) / scale).astype(float).max()
         assert rel <= 2.0 ** -45, (f, np.log2(rel))  # 48 bits less the roundings of the low parts
+
+
+def test_energy_in_pairs_of_floats(run):
+    """1/rho and e - rho u^2 / 2 of the FP32 boundary pass, whose differences to the ambient values matter."""
+    g = np.random.default_rng(3)
+    n = 400000
+    q = np.stack([g.uniform(0.3, 4.0, n), *(g.normal(size=(3, n)) * 10.0 ** g.uniform(-7, 0, n)), g.uniform(3.0, 8.0, n)]).astype(np.float32)
+    v = run(3, q, None, 4).astype(np.longdouble)
+    Q = q.astype(np.longdouble)
+    assert np.abs(((v[0] + v[1]) * Q[0] - 1).astype(float)).max() <= 2.0 ** -46  # the last bit of the low part
+    e = Q[4] - (Q[1] ** 2 + Q[2] ** 2 + Q[3] ** 2) / (2 * Q[0])
+    scale = Q[4] + (Q[1] ** 2 + Q[2] ** 2 + Q[3] ** 2) / (2 * Q[0])
+    assert np.abs(((v[2] + v[3] - e) / scale).astype(float)).max() <= 2.0 ** -44  # five pair operations
