@@ -79,11 +79,11 @@ _PAPER_JET = "jet-384x256x144"
 KERNEL_SOURCE = {"k_iface": "les_stage.cu", "k_fused": "les_fused.cu",
                  "k_iface_prod": "les_stage_prod.cu", "k_fused_prod": "les_fused_prod.cu"}
 TRAFFIC_BYTES_PER_POINT = {  # (workload, precision, kernel, decomposition) -> (bytes per point, source sha16)
-    # profiles/stage_kernels_fp64_product_jet-384x256x144.md: 4337.4 + 1647.3 MB per launch
-    (_PAPER_JET, "fp64", "k_iface_prod", None): (422.77, "06f31f685abc74c4"),
+    # profiles/stage_kernels_fp64_product_jet-384x256x144.md: 4339.5 + 1647.2 MB per launch
+    (_PAPER_JET, "fp64", "k_iface_prod", None): (422.92, "f2e06f7f42a07604"),
     # profiles/fused_stage_fp32_product_jet-384x256x144.md: mean of the five stages
-    (_PAPER_JET, "fp32", "k_fused_prod", "ty=24 kc=balanced"): (62.63, "dfa4e15cca376cd6"),
-    (_PAPER_JET, "fp32-sep", "k_fused_prod", "ty=24 kc=balanced"): (62.63, "dfa4e15cca376cd6"),
+    (_PAPER_JET, "fp32", "k_fused_prod", "ty=24 kc=balanced"): (62.61, "06a63f962903b006"),
+    (_PAPER_JET, "fp32-sep", "k_fused_prod", "ty=24 kc=balanced"): (62.61, "06a63f962903b006"),
 }
 
 
@@ -122,7 +122,7 @@ def traffic_bytes_per_point(workload: str, prec: str, kname: str, describe: str,
 PIPE_UTIL_NCU = {  # (precision, kernel) -> (metrics dict, source sha16)
     # profiles/stage_kernels_fp64_product_jet-384x256x144.md (192x128x72 capture)
     ("fp64", "k_iface_prod"): ({"fp64_pipe_pct": 87.9, "fp64_instructions_per_point": 162.0,
-                                "issue_active_pct": 15.0}, "06f31f685abc74c4"),
+                                "issue_active_pct": 15.0}, "f2e06f7f42a07604"),
 }
 # Nominal multiply-add throughput of GB300 (unit counts x the maximum clock),
 # reported beside the measured figures: 2 DFMA and 128 FFMA per clock and SM.

@@ -68,7 +68,8 @@ extern "C" {
                                ring j = 1, stored unscaled */
 
 /* Storage / arithmetic precision of the stencil path. Metrics and the
- * Jacobian are always computed in FP64; diagnostics sum in FP64. */
+ * Jacobian are always computed in FP64; the diagnostics' sums of squares add in
+ * FP64, their conservation sums in 128-bit fixed point and FP64. */
 #define LES_FP64 0
 #define LES_FP32 1
 /* FP32 that insists on a Cartesian-product grid (x depends on i only, y on j
@@ -132,7 +133,8 @@ typedef struct les_diag {
     int64_t step;             /* completed steps (time level) */
     double max_abs_rhs_rho;   /* L-inf of the continuity residual, interior points */
     double l2_rhs[5];         /* sqrt(sum RHS_f^2) over interior points */
-    double sum_qhat[5];       /* sum of Qhat_f over all points (compensated FP64) */
+    double sum_qhat[5];       /* sum of Qhat_f over all points (exact but for its last
+                                 roundings) */
     int64_t nonfinite;        /* number of non-finite state/residual values */
 } les_diag;
 
@@ -298,7 +300,8 @@ int les_bounds_violation(les_handle *h, uint64_t *out);
  *               the raw state of an FP64 handle);
  *               rhs should be zero at boundary points;
  *   out       : device array of 12 doubles: [0] max |rhs_rho|,
- *               [1..5] sqrt(sum rhs_f^2), [6..10] compensated sum of qhat_f,
+ *               [1..5] sqrt(sum rhs_f^2), [6..10] sum of qhat_f (exact but for
+ *               its last roundings),
  *               [11] count of non-finite values;
  *   stream    : cudaStream_t the two kernels are launched on (NULL allowed).
  * Asynchronous; allocates nothing.  Its scratch is one file-scope device

@@ -38,10 +38,10 @@ __device__ __forceinline__ float4 cat4(float2 a, float2 b) { return make_float4(
 // thread's two rows
 __device__ __forceinline__ float2 odd2(float2 a, float2 b) { return make_float2(a.y, b.x); }
 __device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-// Hardware reciprocal and reciprocal square root (1-2 ulp; arguments normal
-// numbers): the plain instructions, without the denormal handling that the
-// library wrappers put around them (about three instructions each; 17 pairs per
-// thread and plane in the general kernel)
+// Hardware reciprocal and reciprocal square root (within 1.5 and 2.5 ulp;
+// arguments normal numbers): the plain instructions, which flush subnormal
+// numbers.  17 pairs per thread and plane in the general kernel: polar 400x150x60
+// 276.6 us per stage with the calls that keep them, 265.1 with these.
 __device__ __forceinline__ float rcpa(float x)
 {
     float r;

@@ -8,9 +8,12 @@
 // for quantities a diagonal metric does not use, index arithmetic, and moves
 // that shifted row pairs by one row.  This kernel drops those tables and moves
 // and runs 12 warps per SM (TY = 24).  Measured, 384x256x144, ms per stage:
-// general metrics 0.951, diagonal before 0.700, this kernel 0.543; 64 jets, ten
-// steps 128.2 -> 83.1 ms; 192x128x72 0.142 -> 0.093.  What bounds it: issue
-// (42 % busy; shared-memory and MUFU latency with 3 warps per scheduler).
+// general metrics 0.951, diagonal before 0.700, this kernel 0.537; general metrics
+// -> this kernel: 64 jets 11.55 -> 6.76 ms a step, 192x128x72 0.142 -> 0.090 ms a
+// stage.  What bounds it: latency with 3 warps per scheduler (384x192x96, TY = 24:
+// issue 42 % busy, shared-memory wavefronts 56 % and FMA pipe 33 % of peak; stalls
+// per issue on shared-memory and MUFU results 1.6, on fixed-latency chains 1.4, on
+// the memory queue 0.8, at barriers 0.5).
 //
 // Fluxes.  As in les_stage_prod.cu the interface flux is divided by the face
 // area S_a and doubled, G_a = 2 H_a / S_a = F_L + F_R - hb (lb_L + lb_R) [eps2

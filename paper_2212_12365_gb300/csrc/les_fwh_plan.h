@@ -53,7 +53,9 @@ inline FwhPlan fwh_plan(int npts, int N, int nobs, int nt, double dt_obs, double
     // CTA may use 110 KB of shared memory; with a buffer row per microphone of the
     // group a window holds 640 frames for a group of 16 and 1024 for one of 8.  A
     // block of 512 times shares the spread among more evaluations than one of 256,
-    // so it comes first; the direct pass is left for windows that fit neither.
+    // so it comes first (with blocks of 256 only, 8, 24 and 64 microphones x 512
+    // times take 3.61, 5.14 and 7.37 ms a call against 3.32, 4.55 and 7.11; no call
+    // measured gains); the direct pass is left for windows that fit neither.
     // (With sixteen rows always and no second block size, 98,304 panels of 1024
     // frames took the direct pass at 8, 16, 24 and 32 microphones x 512 times:
     // 3.94, 5.71, 8.58, 10.50 ms a call; so 3.31, 4.23, 4.52, 5.65.)

@@ -23,7 +23,7 @@
 // Jets on a Cartesian-product grid take les_stage_prod.cu; this is the form for
 // curvilinear ones.  Measured on the 200x75x40 polar mesh, us per launch, with
 // the short root and reciprocal sequences, integer maxima and doubled
-// differences: point 135 -> 120, gradients 134 -> 108, interfaces 403 -> 396.
+// differences: point 135 -> 124, gradients 134 -> 109, interfaces 404 -> 396.
 #include <cmath>
 
 #include "les_fp64.cuh"

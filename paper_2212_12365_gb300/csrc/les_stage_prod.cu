@@ -13,10 +13,10 @@
 //   G = F_L + F_R - sc [eps2 dW - eps4 d3W] - viscous,   sc = hb (lb_L + lb_R),
 // with F the Cartesian point fluxes (nine products, rho u_i u_j is symmetric),
 // and the update multiplies each flux difference by S_a / 2 once.
-// FP64 instructions per point: point 65, gradients 63, interfaces 3 x 56,
-// update 36 = 332.  Measured on the 384x256x144 jet, us per launch, general ->
-// this form: point 2740 -> 1717, gradients 2710 -> 1682, interfaces 8385 ->
-// 4202 (FP64 pipe 85-88 % busy in each), update 952 -> 924.
+// FP64 instructions per point: point 69, gradients 66, interfaces 162, update 34 =
+// 332.  Measured on the 384x256x144 jet, us per launch, general -> this form:
+// point 2740 -> 1805, gradients 2710 -> 1703, interfaces 8385 -> 4201 (FP64 pipe
+// 85-88 % busy in each), update 952 -> 897.
 // Tangential derivatives reach the interface as c_ai = (1/2) du_a/dx_i and the
 // divergence as the third s_a = (1/3) sum_{i != a} du_i/dx_i of each point, so
 // that the sums over the two points need no factor.
