@@ -12,9 +12,9 @@
 // what reaches below it is kept in a double of its own, so that large values may
 // cancel without a trace (a test holds the sums to the exactly rounded ones).
 // The sums of squares stay in FP64 (one multiply-add per value).
-// Measured: 14,155,776 points 2098 -> 244 us (4.6 TB/s; 236 without the tails);
-// les_get_diagnostics of a 192x128x72 FP32 jet about 1.0 ms less per call (most of
-// it the final pass).
+// Measured: 14,155,776 points 2098 -> 219 us (5.2 TB/s), 1,000,000 908 -> 49, one
+// point 27 -> 22; les_get_diagnostics of a 192x128x72 FP32 jet about 1.0 ms less
+// per call (most of it the final pass).
 #pragma once
 
 #include "les_internal.cuh"
@@ -179,20 +179,28 @@ template <typename Load> __device__ __forceinline__ void sum_block(long long ste
     }
     bad = __reduce_add_sync(0xffffffffu, bad);
     nf = __reduce_or_sync(0xffffffffu, nf);
+    // lane f takes field f, so that the five conversions run at once (one after the
+    // other, each in its own lane, they took 11 us of every call: one point 33 us)
+    SumFx own;
+    double l2o = 0.0, tail = 0.0;
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
         fx[f].warp_reduce();
-        double tail = tails[f][threadIdx.x];
+        double t = tails[f][threadIdx.x];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane == f) {
-            double s, c;
-            fx[f].value(s, c);
-            c += tail;
-            sh[1 + f][w] = l2[f];
-            sh[6 + f][w] = (nf >> f) & 1 ? __longlong_as_double(0x7ff8000000000000ll) : s;
-            sh[11 + f][w] = c;
+            own = fx[f];
+            l2o = l2[f];
+            tail = t;
         }
+    }
+    if (lane < 5) {
+        double s, c;
+        own.value(s, c);
+        sh[1 + lane][w] = l2o;
+        sh[6 + lane][w] = (nf >> lane) & 1 ? __longlong_as_double(0x7ff8000000000000ll) : s;
+        sh[11 + lane][w] = c + tail;
     }
     if (lane == 0) {
         sh[0][w] = mx;
