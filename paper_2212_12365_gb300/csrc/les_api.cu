@@ -523,6 +523,10 @@ static int set_fused_tiling(les_handle *h, int fi, int ty, int kc)
         one[j] = F;
         one[j].item0 = 0;
         one[j].tile0 = 0;
+        if (h->njets > 1) { // a jet of a batch alone (its residual): balanced, see fused_launch_form
+            one[j].kc = 0;
+            one[j].nkc = out_len(J, 2);
+        }
     }
     M.ty = ty;
     M.balanced = kc == 0 ? 1 : (kc < 0 ? 2 : 0);
@@ -573,8 +577,12 @@ static void fused_launch_form(les_handle *h, int fi, int jet, int src, int dst, 
     const JetDev<float> *jets = (const JetDev<float> *)h->d_jets;
     const FusedJet *fj = jet < 0 ? M.d_fj : M.d_fj1 + jet;
     const int nj = jet < 0 ? h->njets : 1;
-    const int items = jet < 0 ? M.items : items_of(M.fj[jet]);
-    const int tiles = jet < 0 ? M.tiles : M.fj[jet].nbx * M.fj[jet].nby;
+    // A jet of a batch by itself takes the balanced form: the decomposition that
+    // suits the whole batch leaves most SMs idle on one of its jets (residual and
+    // read-back of a 110x37x43 jet 138 us with the batch's chunks of 16 planes, 99 so).
+    const int bal = jet >= 0 && h->njets > 1 ? 1 : M.balanced;
+    const int items = jet < 0 ? M.items : items_of(M.fj1[jet]);
+    const int tiles = jet < 0 ? M.tiles : M.fj1[jet].nbx * M.fj1[jet].nby;
     const int grid = std::max(1, std::min(items, h->nsm * M.cps[M.ty / 8 - 1]));
     const double *dt = h->d_dt;
     if (jet >= 0) {
@@ -584,7 +592,7 @@ static void fused_launch_form(les_handle *h, int fi, int jet, int src, int dst, 
     // a single jet's table entries travel as kernel parameters
     const JetDev<float> *j1 = nj == 1 ? &h->jd32[jet < 0 ? 0 : jet] : nullptr;
     const FusedJet *f1 = nj == 1 ? (jet < 0 ? &M.fj[0] : &M.fj1[jet]) : nullptr;
-    const FusedLaunch a{jets, fj, nj, items, tiles, src, dst, stage, dt, rhs_only, M.balanced, h->stage_wait_limit};
+    const FusedLaunch a{jets, fj, nj, items, tiles, src, dst, stage, dt, rhs_only, bal, h->stage_wait_limit};
     if (fi == 1) launch_fused_prod(M.ty, a, grid, j1, f1, st);
     else launch_fused(M.ty, a, grid, j1, f1, st);
 }
