@@ -10,8 +10,8 @@
 // residual: t = x y0 rounded, r = x - t^2 (exact but for its last bit), sqrt(x) =
 // t + r y0 (1/2 + 3 e/8), so that the rounding of t does not reach the result:
 // six operations, within 0.53 ulp.  (As t (1 + e/2 + 3 e^2/8), five operations,
-// it was off by up to 0.76 ulp; ten FP64 steps took 3116 us on 48x32x32 and 34.05
-// ms on the polar 200x75x40 with that form and take 3144 us and 34.32 ms.)
+// it was off by up to 0.76 ulp; the sixth operation costs ten FP64 steps 28 us of
+// 3120 on 48x32x32 and 0.27 ms of 34.3 on the polar 200x75x40.)
 // Comparisons of non-negative numbers go to the integer pipe.
 #pragma once
 
